@@ -109,6 +109,46 @@ void make_tp_table(int N, std::vector<double>& out) {
   }
 }
 
+// The FP64 form's tables of an axis of length N <= 8192 (csl_fix.cuh): half
+// sines and pass tables in signed digits.  Sines and cosines are evaluated
+// for one eighth of the circle and the rest follows by symmetry.
+void make_fix_tables(int N, std::vector<int2>& hs, std::vector<fxw>& tp) {
+  // quarter-wave cosine of 2 N points, cos(pi m / N), m = 0 .. N/2
+  std::vector<long long> qc(N / 2 + 1);
+  for (int m = 0; m <= N / 4; ++m) {
+    const FxRoot r = fx_root(m, 2 * N);
+    qc[m] = r.c;
+    qc[N / 2 - m] = r.s;
+  }
+  hs.resize(N / 2 + 1);
+  for (int j = 0; j <= N / 2; ++j) {
+    const FxDigits d = fx_digits(qc[N / 2 - j] >> 1);
+    hs[j] = make_int2(d.h, d.l);
+  }
+  tp.clear();
+  for (int v = 0; v <= (N == 512 || N == 1024 ? 2 : 0); v += 2) {
+    const FixRadices f = fix_radices_of(N, v);
+    int ls = f.r[0];
+    for (int p = 1; p < f.np; ++p) {
+      const int n = ls * f.r[p];
+      for (int e = 0; e < n; ++e) {
+        // exp(-2 pi i m / N) = cos(pi 2m / N) - i sin(pi 2m / N)
+        const int m2 = 2 * (int)((long)(e / ls) * (e % ls) % n * (N / n));
+        const int quad = m2 / (N / 2), r = m2 - quad * (N / 2);
+        long long c = qc[r], sn = qc[N / 2 - r];
+        for (int i = 0; i < quad; ++i) {
+          const long long t = c;
+          c = -sn;
+          sn = t;
+        }
+        const FxDigits dc = fx_digits(fx_quant(c, kFxTw)), ds = fx_digits(fx_quant(-sn, kFxTw));
+        tp.push_back(make_int4(dc.h, dc.l, ds.h, ds.l));
+      }
+      ls = n;
+    }
+  }
+}
+
 }  // namespace
 
 struct csl_plan {
@@ -211,7 +251,7 @@ cudaError_t set_attrs_once() {
 // shared memory fits ~100 KB (two or more CTAs per SM).
 template <typename T>
 void choose_cta(PassCfg& c, int want_threads) {
-  const int tpl = pass_tpl(c.N, c.wide);
+  const int tpl = pass_tpl<T>(c.N, c.wide);
   int threads = want_threads;
   while (threads > 32 && threads > tpl && pass_smem<T>(c.N, c.wide, threads / tpl) > 100 * 1024) threads >>= 1;
   c.lines = threads / tpl;
@@ -236,13 +276,13 @@ void config_row(PassCfg& c, int n, int nrows) {
   if (pass_is_big(c.N)) {  // one CTA of all the line's lanes per row
     c.wide = 3;
     c.lines = 1;
-    c.L.threads = pass_tpl(c.N, 3);
+    c.L.threads = pass_tpl<T>(c.N, 3);
     c.L.smem = pass_smem<T>(c.N, 3, 1);
     c.L.blocks = nrows < kSMs * 8 ? nrows : kSMs * 8;
     return;
   }
   int threads = 256;
-  const int tpl = pass_tpl(c.N, c.wide);
+  const int tpl = pass_tpl<T>(c.N, c.wide);
   // few rows: smaller CTAs so that every SM gets work
   while (threads > 32 && threads / tpl > 1 && (nrows + threads / tpl - 1) / (threads / tpl) < 2 * kSMs) threads >>= 1;
   choose_cta<T>(c, threads);
@@ -270,13 +310,13 @@ void config_strided(PassCfg& c, int n, int ncols, int nouter, long outer_stride,
   if (pass_is_big(c.N)) {  // one column per CTA
     c.wide = 3;
     c.lines = 1;
-    c.L.threads = pass_tpl(c.N, 3);
+    c.L.threads = pass_tpl<T>(c.N, 3);
     c.L.smem = pass_smem<T>(c.N, 3, 1);
     const long tiles = (long)ncols * nouter;
     c.L.blocks = (int)(tiles < kMaxRedBlocks ? tiles : kMaxRedBlocks);
     return;
   }
-  const int tpl = pass_tpl(c.N, c.wide);
+  const int tpl = pass_tpl<T>(c.N, c.wide);
   int threads = 256;
   if (want_lines > 0) {
     int l = 1;
@@ -304,7 +344,7 @@ RowArgs<T> row_args(csl_plan* P) {
   a.nrows = P->row.nouter;
   a.tw = (const typename C2<T>::t*)P->tw[0];
   a.hs = (const T*)P->hs[0];
-  a.tp = (const typename C2<T>::t*)P->tp[0] + (P->row.wide ? line_tp_size(P->row.N, false) : 0);
+  a.tp = (const typename C2<T>::t*)P->tp[0] + pass_tp_offset<T>(P->row.N, P->row.wide);
   return a;
 }
 
@@ -323,7 +363,7 @@ StridedArgs<T> strided_args(csl_plan* P, const PassCfg& c, int axis) {
   a.line_stride = c.line_stride;
   a.tw = (const typename C2<T>::t*)P->tw[axis];
   a.hs = (const T*)P->hs[axis];
-  a.tp = (const typename C2<T>::t*)P->tp[axis] + (c.wide ? line_tp_size(c.N, false) : 0);
+  a.tp = (const typename C2<T>::t*)P->tp[axis] + pass_tp_offset<T>(c.N, c.wide);
   a.data = (typename C2<T>::t*)P->T;
   a.sine_tc = P->sine_tc[axis];
   return a;
@@ -694,7 +734,7 @@ std::mutex g_tune_mu;
 template <typename T>
 bool make_candidate(const PassCfg& c, int kind, int w, int lines, PassCfg& cand) {
   if (w < 0 || w >= pass_num_variants(c.N) || lines < 1 || (lines & (lines - 1))) return false;
-  const int tpl = pass_tpl(c.N, w);
+  const int tpl = pass_tpl<T>(c.N, w);
   if (lines * tpl < 32 || lines * tpl > 256) return false;
   cand = c;
   cand.wide = w;
@@ -755,7 +795,7 @@ cudaError_t tune_pass(csl_plan* P, PassCfg& c, int kind, cudaEvent_t* ev, const 
   double best_ms = 1e30;
   double ms[8];
   cudaError_t e = cudaSuccess;
-  for (int w = 0; w < pass_num_variants(keep.N) && e == cudaSuccess; ++w) {
+  for (int w = pass_first_variant<T>(keep.N); w < pass_num_variants(keep.N) && e == cudaSuccess; ++w) {
     for (int lines = 1; lines <= 256 && e == cudaSuccess; lines <<= 1) {
       PassCfg cand;
       if (!make_candidate<T>(keep, kind, w, lines, cand)) continue;
@@ -1031,7 +1071,8 @@ csl_status csl_plan_create(csl_plan** out, int dim, const int64_t n[3], const do
   }
   const long M = P->M;
   const int nx = P->n[0], ny = P->n[1], nz = P->n[2];
-  const size_t tsz = o.precision != CSL_PREC_FP64 ? sizeof(float) : sizeof(double);
+  const bool fp64 = o.precision == CSL_PREC_FP64;
+  const size_t tsz = fp64 ? sizeof(double) : sizeof(float);
   long nface[3];
   nface[0] = (long)nz * ny * (nx + 1);
   nface[1] = (long)nz * (ny + 1) * nx;
@@ -1057,7 +1098,7 @@ csl_status csl_plan_create(csl_plan** out, int dim, const int64_t n[3], const do
     P->mu_f[d] = (float*)dalloc(P, (size_t)P->n[d] * 4, &err);
     P->tw[d] = dalloc(P, (size_t)(N / 2) * 2 * tsz, &err);
     P->hs[d] = dalloc(P, (size_t)(N / 2 + 1) * tsz, &err);
-    P->tp[d] = dalloc(P, (size_t)(line_tp_size(N, false) + line_tp_size(N, true) + 1) * 2 * tsz, &err);
+    P->tp[d] = dalloc(P, (size_t)((fp64 ? pass_tp_total<double>(N) : pass_tp_total<float>(N)) + 1) * 2 * tsz, &err);
   }
   P->b = (double2*)dalloc(P, M * 16, &err);
   P->x = (double2*)dalloc(P, M * 16, &err);
@@ -1181,6 +1222,17 @@ csl_status csl_plan_create(csl_plan** out, int dim, const int64_t n[3], const do
       mu[k - 1] = 4.0 / (P->h[d] * P->h[d]) * sn * sn;
       muf[k - 1] = (float)mu[k - 1];
     }
+    err = cudaMemcpy(P->mu_d[d], mu.data(), nd * 8, cudaMemcpyHostToDevice);
+    if (err == cudaSuccess) err = cudaMemcpy(P->mu_f[d], muf.data(), nd * 4, cudaMemcpyHostToDevice);
+    if (fp64 && N <= 8192) {  // 64-bit fixed-point tables
+      std::vector<int2> hsx;
+      std::vector<fxw> tpx;
+      make_fix_tables(N, hsx, tpx);
+      if (err == cudaSuccess) err = cudaMemcpy(P->hs[d], hsx.data(), hsx.size() * sizeof(int2), cudaMemcpyHostToDevice);
+      if (err == cudaSuccess && !tpx.empty())
+        err = cudaMemcpy(P->tp[d], tpx.data(), tpx.size() * sizeof(fxw), cudaMemcpyHostToDevice);
+      continue;
+    }
     std::vector<double> twd(N), hsd(N / 2 + 1);
     for (int m = 0; m < N / 2; ++m) {
       twd[2 * m] = cos(2.0 * M_PI * (double)m / N);
@@ -1188,31 +1240,18 @@ csl_status csl_plan_create(csl_plan** out, int dim, const int64_t n[3], const do
     }
     for (int j = 0; j <= N / 2; ++j) hsd[j] = 0.5 * sin(M_PI * (double)j / N);
     hsd[N / 2] = 0.5;
-    std::vector<double> tpd;
-    make_tp_table(N, tpd);
-    const size_t ntp = tpd.size();
-    if (ntp) {
-      if (o.precision != CSL_PREC_FP64) {
-        std::vector<float> tpf(ntp);
-        for (size_t i = 0; i < ntp; ++i) tpf[i] = (float)tpd[i];
-        err = cudaMemcpy(P->tp[d], tpf.data(), ntp * 4, cudaMemcpyHostToDevice);
-      } else {
-        err = cudaMemcpy(P->tp[d], tpd.data(), ntp * 8, cudaMemcpyHostToDevice);
-      }
-      if (err != cudaSuccess) break;
-    }
-    err = cudaMemcpy(P->mu_d[d], mu.data(), nd * 8, cudaMemcpyHostToDevice);
-    if (err == cudaSuccess) err = cudaMemcpy(P->mu_f[d], muf.data(), nd * 4, cudaMemcpyHostToDevice);
-    if (o.precision != CSL_PREC_FP64) {
-      std::vector<float> twf(N), hsf(N / 2 + 1);
-      for (int i = 0; i < N; ++i) twf[i] = (float)twd[i];
-      for (int j = 0; j <= N / 2; ++j) hsf[j] = (float)hsd[j];
-      if (err == cudaSuccess) err = cudaMemcpy(P->tw[d], twf.data(), N * 4, cudaMemcpyHostToDevice);
-      if (err == cudaSuccess) err = cudaMemcpy(P->hs[d], hsf.data(), (N / 2 + 1) * 4, cudaMemcpyHostToDevice);
-    } else {
+    if (fp64) {  // lines of 16384 points: FP64 arithmetic on two-CTA clusters
       if (err == cudaSuccess) err = cudaMemcpy(P->tw[d], twd.data(), N * 8, cudaMemcpyHostToDevice);
       if (err == cudaSuccess) err = cudaMemcpy(P->hs[d], hsd.data(), (N / 2 + 1) * 8, cudaMemcpyHostToDevice);
+      continue;
     }
+    std::vector<double> tpd;
+    make_tp_table(N, tpd);
+    std::vector<float> tpf(tpd.begin(), tpd.end()), twf(twd.begin(), twd.end()), hsf(hsd.begin(), hsd.end());
+    if (err == cudaSuccess && !tpf.empty())
+      err = cudaMemcpy(P->tp[d], tpf.data(), tpf.size() * 4, cudaMemcpyHostToDevice);
+    if (err == cudaSuccess) err = cudaMemcpy(P->tw[d], twf.data(), N * 4, cudaMemcpyHostToDevice);
+    if (err == cudaSuccess) err = cudaMemcpy(P->hs[d], hsf.data(), (N / 2 + 1) * 4, cudaMemcpyHostToDevice);
   }
   // per-mode scale of P^{-1} (Eq. 4) and the extremes of its eigenvalues
   if (err == cudaSuccess) {

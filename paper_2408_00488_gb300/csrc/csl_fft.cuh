@@ -28,6 +28,7 @@
 // conflicts.
 #pragma once
 #include "csl_common.cuh"
+#include "csl_fix.cuh"
 
 namespace csl {
 
@@ -422,23 +423,47 @@ __device__ __forceinline__ void dst_line_wide(typename C2<T>::t* a, int t, const
 // line; V = 1, 2: wide path with 64 or 128 lanes per line.
 //   TPL       lanes per line (lines = threadIdx / TPL)
 //   LS        shared-memory line stride (complex elements)
-//   TP        size of the extra twiddle table (four-step [k1][g] table, or the
-//             wide path's per-pass tables; 0 for single-thread lines)
-//   BLOCK_SYNC whether the transform uses CTA-wide barriers
+//   SCRATCH   complex slots per line for the scan
+//   Tables    what the transform reads, and its bytes of shared memory
 // ---------------------------------------------------------------------------
 template <typename T, int N, int V = 0>
 struct LineDst;
 
+// tables of a line transform: half-length twiddles, half sines, extra twiddles
+template <typename T>
+struct LineTab {
+  const typename C2<T>::t* tw;
+  const T* hs;
+  const typename C2<T>::t* tp;
+};
+
+// copied into shared memory (block-wide): twiddles | half sines | extra twiddles
+template <typename T, int N, int NTP>
+struct SmemTables {
+  typedef typename C2<T>::t c_t;
+  static constexpr size_t kHs = (size_t)(N / 2) * sizeof(c_t), kTp = kHs + (((size_t)(N / 2 + 1) * sizeof(T) + 15) / 16) * 16,
+                          kBytes = kTp + (size_t)NTP * sizeof(c_t);
+  static __device__ __forceinline__ LineTab<T> load(unsigned char* smem, const c_t* tw, const T* hs, const c_t* tp) {
+    c_t* s_tw = (c_t*)smem;
+    T* s_hs = (T*)(smem + kHs);
+    c_t* s_tp = (c_t*)(smem + kTp);
+    for (int i = threadIdx.x; i < N / 2; i += blockDim.x) s_tw[i] = tw[i];
+    for (int i = threadIdx.x; i <= N / 2; i += blockDim.x) s_hs[i] = hs[i];
+    for (int i = threadIdx.x; i < NTP; i += blockDim.x) s_tp[i] = tp[i];
+    return {s_tw, s_hs, s_tp};
+  }
+};
+
 template <typename T, int N>
 struct LineDst<T, N, 0> {
   typedef typename C2<T>::t c_t;
-  enum { TPL = DstShape<N>::TPL, LS = dst_line_stride<N>(), BLOCK_SYNC = 0,
-         TP = DstShape<N>::R2 == 1 ? 0 : N, GLOBAL_TABLES = 0 };
+  typedef SmemTables<T, N, DstShape<N>::R2 == 1 ? 0 : N> Tables;
+  enum { TPL = DstShape<N>::TPL, LS = dst_line_stride<N>(), SCRATCH = 4 };
   static __device__ __forceinline__ int in_pos(int j) { return j; }
   static __device__ __forceinline__ int out_pos(int m) { return dst_out_pos<N>(m); }
   template <bool PERM_IN>
-  static __device__ __forceinline__ void run(c_t* a, int t, const c_t* tw, const T* hs, const c_t* tp, c_t*) {
-    dst_line<T, N, PERM_IN>(a, t, tw, hs, tp);
+  static __device__ __forceinline__ void run(c_t* a, int t, const LineTab<T>& tb, c_t*) {
+    dst_line<T, N, PERM_IN>(a, t, tb.tw, tb.hs, tb.tp);
   }
   static __device__ __forceinline__ void line_sync() { __syncwarp(); }
 };
@@ -446,14 +471,13 @@ struct LineDst<T, N, 0> {
 template <typename T, int N, int V>
 struct LineDst {
   typedef typename C2<T>::t c_t;
-  enum { TPL = wide_tpl(V), LS = wide_line_stride<N, wide_tpl(V)>(), BLOCK_SYNC = 1, TP = wide_tp_size<N>(),
-         GLOBAL_TABLES = 0 };
+  typedef SmemTables<T, N, wide_tp_size<N>()> Tables;
+  enum { TPL = wide_tpl(V), LS = wide_line_stride<N, wide_tpl(V)>(), SCRATCH = 4 };
   static __device__ __forceinline__ int in_pos(int j) { return wpad(j); }
   static __device__ __forceinline__ int out_pos(int m) { return wide_out_pos<N, TPL>(m); }
   template <bool PERM_IN>
-  static __device__ __forceinline__ void run(c_t* a, int t, const c_t* tw, const T* hs, const c_t* tp,
-                                             c_t* scratch) {
-    dst_line_wide<T, N, TPL, PERM_IN>(a, t, tw, hs, tp, scratch);
+  static __device__ __forceinline__ void run(c_t* a, int t, const LineTab<T>& tb, c_t* scratch) {
+    dst_line_wide<T, N, TPL, PERM_IN>(a, t, tb.tw, tb.hs, tb.tp, scratch);
   }
   static __device__ __forceinline__ void line_sync() { __syncthreads(); }
 };
@@ -580,31 +604,77 @@ __device__ __forceinline__ void dst_line_big(typename C2<T>::t* a, int t, const 
 template <typename T, int N>
 struct LineDst<T, N, 3> {
   typedef typename C2<T>::t c_t;
-  enum { TPL = BigShape<N>::TPL, LS = wide_line_stride<N, BigShape<N>::TPL>(), BLOCK_SYNC = 1, TP = 0,
-         GLOBAL_TABLES = 1 };
+  struct Tables {  // read from global memory through the cache
+    static constexpr size_t kBytes = 0;
+    static __device__ __forceinline__ LineTab<T> load(unsigned char*, const c_t* tw, const T* hs, const c_t* tp) {
+      return {tw, hs, tp};
+    }
+  };
+  // the scan runs in FP64: twice as many T-complex slots
+  enum { TPL = BigShape<N>::TPL, LS = wide_line_stride<N, BigShape<N>::TPL>(), SCRATCH = TPL / 16 };
   static __device__ __forceinline__ int in_pos(int j) { return wpad(j); }
   static __device__ __forceinline__ int out_pos(int m) { return wide_out_pos<N, TPL>(m); }
   template <bool PERM_IN>
-  static __device__ __forceinline__ void run(c_t* a, int t, const c_t* tw, const T* hs, const c_t*, c_t* scratch) {
-    dst_line_big<T, N, PERM_IN>(a, t, tw, hs, scratch);
+  static __device__ __forceinline__ void run(c_t* a, int t, const LineTab<T>& tb, c_t* scratch) {
+    dst_line_big<T, N, PERM_IN>(a, t, tb.tw, tb.hs, scratch);
   }
   static __device__ __forceinline__ void line_sync() { __syncthreads(); }
 };
 
-// Host-side size of the extra twiddle table of length N (matches LineDst::TP).
+// The FP64 form: 64-bit block fixed point (csl_fix.cuh).  The line buffer
+// holds doubles before and after; input and output positions agree.  Tables:
+// half sines and pass tables (signed digits, the sizes of a double and a
+// double2), in shared memory up to N = 1024.
+template <int N, int LANES, bool GLOBAL>
+struct FixDst {
+  typedef FixLine<N, LANES> F;
+  enum { TPL = LANES, LS = fix_line_stride<N>(), SCRATCH = 2 * (LANES / 32 > 4 ? LANES / 32 : 4) };
+  struct Tab {
+    const int2* hs;
+    const fxw* tp;
+  };
+  struct Tables {
+    static constexpr int kTpN = fix_table_entries<N, LANES>();
+    static constexpr size_t kTp = (((size_t)(N / 2 + 1) * 8 + 15) / 16) * 16,
+                            kBytes = GLOBAL ? 0 : kTp + (size_t)kTpN * sizeof(fxw);
+    static __device__ __forceinline__ Tab load(unsigned char* smem, const double2*, const double* hs,
+                                               const double2* tp) {
+      if constexpr (GLOBAL) return {(const int2*)hs, (const fxw*)tp};
+      int2* s_hs = (int2*)smem;
+      fxw* s_tp = (fxw*)(smem + kTp);
+      for (int i = threadIdx.x; i <= N / 2; i += blockDim.x) s_hs[i] = ((const int2*)hs)[i];
+      for (int i = threadIdx.x; i < kTpN; i += blockDim.x) s_tp[i] = ((const fxw*)tp)[i];
+      return {s_hs, s_tp};
+    }
+  };
+  static __device__ __forceinline__ int in_pos(int j) { return fpad(j); }
+  static __device__ __forceinline__ int out_pos(int m) { return fpad(m); }
+  // scr: SCRATCH slots per line
+  template <bool PERM_IN>
+  static __device__ __forceinline__ void run(double2* a, int t, const Tab& tb, double2* scr) {
+    FixNoPost none;
+    run_post(a, t, tb, scr, none);
+  }
+  template <typename POST>
+  static __device__ __forceinline__ void run_post(double2* a, int t, const Tab& tb, double2* scr, POST& post) {
+    F::run(a, t, tb.hs, tb.tp, scr + SCRATCH * (threadIdx.x / LANES), post);
+  }
+  static __device__ __forceinline__ void line_sync() {
+    if constexpr (LANES > 1) fx_line_sync(LANES);
+  }
+};
+// lanes per line: 8 to 16 values a lane; N = 512 and 1024 have no
+// warp-per-line variant (32 values a lane spill), 0 stands for 1 there
+template <int N>
+struct LineDst<double, N, 0> : FixDst<N, N == 32 ? 4 : N >= 512 ? 64 : DstShape<N>::TPL, false> {};
+template <int N, int V>
+struct LineDst<double, N, V> : FixDst<N, wide_tpl(V), false> {};
+template <int N>
+struct LineDst<double, N, 3> : FixDst<N, BigShape<N>::TPL, true> {};
+
+// Host-side size of the extra twiddle table of length N in the FP32 forms.
 __host__ __device__ constexpr int line_tp_size(int N, int wide) {
   return wide ? (N >= 1024 ? wide_tp_size<1024>() : N >= 512 ? wide_tp_size<512>() : 0) : (N >= 64 ? N : 0);
-}
-
-// Copy the transform tables of length N into shared memory (block-wide).
-template <typename T>
-__device__ __forceinline__ void load_tables(typename C2<T>::t* s_tw, T* s_hs, typename C2<T>::t* s_tp,
-                                            const typename C2<T>::t* g_tw, const T* g_hs,
-                                            const typename C2<T>::t* g_tp, int N, int ntp) {
-  const int H = N >> 1;
-  for (int i = threadIdx.x; i < H; i += blockDim.x) s_tw[i] = g_tw[i];
-  for (int i = threadIdx.x; i <= H; i += blockDim.x) s_hs[i] = g_hs[i];
-  for (int i = threadIdx.x; i < ntp; i += blockDim.x) s_tp[i] = g_tp[i];
 }
 
 }  // namespace csl

@@ -1,0 +1,685 @@
+// FP64-accurate sine transform of one line in 64-bit block fixed point.
+//
+// GB300 issues FP64 at 2 lanes per SM and clock (measured 1.6 to 2, one
+// dependent operation every 67 clocks) but 64-bit integer sums at about 41 and
+// 32 x 32 -> 64 bit products at 60, so an FFT in FP64 arithmetic is bound by
+// that one pipe.  Here the line is scaled by one power of two, held as 64-bit
+// integers, and transformed with integer butterflies.  Sums are exact; a
+// product is rounded once.  Relative to the line's norm the error is below
+// that of the FP64 butterflies, whose every operation rounds to 53 bits.
+//
+// The algorithm is that of csl_fft.cuh (one length-N complex FFT per line,
+// y_j = h_j (z_j + z_{N-j}) + (z_j - z_{N-j})/4, the C / S split and the
+// prefix sum), as a Stockham FFT with radices R0 .. R3.
+//
+// Scales.  E = largest exponent of the line, so |re|, |im| < 2^(E-1022).
+//   pass 1         values times 2^(S1 - (E-1022)), S1 chosen so that R0 sqrt(2) 2^S1 < 2^62
+//   later passes   shifted right by sh_p while the twiddle is applied, only as
+//                  far as needed: every value of pass p is bounded by both
+//                  sqrt(2) max|z| R0..Rp and by the line's sum of |re| + |im|
+//                  (the bound of every partial DFT sum, and of the result:
+//                  sum_j |y_j| <= sum_j |z_j| because max(s_j, 1/2) <= 1)
+// so nothing overflows for any input, a line of one spike keeps S1 bits, and
+// the rounding of the early passes, which later passes amplify, happens at
+// the finer scale.  The split and the prefix sum only add, modulo 2^64, and
+// their results fit.
+//
+// Measured on a GB300, FP64 form, per iteration of MINRES: n = 1023 in 2D, x
+// pass with the Lanczos step 124.6 us in FP64 arithmetic, 36.3 here; MID pass
+// 252.5 and 72.2; inverse x pass 119.0 and 35.1; whole iteration 524 and 178.
+// n = 127 in 3D 1067 and 413 us; n = 4095 9297 and 3237.  Error of one line
+// against long double: 0.05 to 0.9 times that of the FP64 butterflies for
+// random, smooth, decaying and constant lines of 4 to 8192 points, about the
+// same for a spike of 4096.  What bounds it now is latency: 11 to 16 warps per
+// SM (registers and shared memory hold the lines), integer pipe 30% busy.
+//
+// A line with an infinity or NaN returns NaN everywhere (the FP64 butterflies
+// spread it over the line too); a zero line returns zeros.
+#pragma once
+#include "csl_common.cuh"
+
+#include <climits>
+
+namespace csl {
+
+typedef longlong2 fx2;  // (re, im)
+typedef int4 fxw;       // twiddle: signed 32-bit digits re_hi, re_lo, im_hi, im_lo (value hi 2^32 + lo)
+
+// fractional bits of the twiddle tables: products are taken back by
+// kFxTw + sh <= 64 bits, i.e. one 32-bit funnel shift by kFxTw - 32 + sh <= 32
+constexpr int kFxTw = 61;
+constexpr int kFxMaxShift = 3;
+
+// ---- constants -----------------------------------------------------------------
+__host__ __device__ constexpr unsigned long long fx_mulhi(unsigned long long a, unsigned long long b) {
+  const unsigned long long al = a & 0xffffffffull, ah = a >> 32, bl = b & 0xffffffffull, bh = b >> 32;
+  const unsigned long long t = al * bl, u = ah * bl + (t >> 32), v = al * bh + (u & 0xffffffffull);
+  return ah * bh + (u >> 32) + (v >> 32);
+}
+
+struct FxRoot {
+  long long c, s;  // cos, sin with 62 fractional bits
+};
+
+// cos and sin of 2 pi num / den (den a power of two, 0 <= num < den) to within
+// a few units of 2^-62: reduction to [0, pi/4] by exact symmetries, then the
+// Taylor series by Horner's rule in fixed point (the first term left out is
+// (pi/4)^20 / 20! < 2^-67).
+__host__ __device__ constexpr FxRoot fx_root(int num, int den) {
+  long long n = num, d = den;
+  int ld = 0;
+  while (d < 8) {
+    n *= 2;
+    d *= 2;
+  }
+  while ((1ll << ld) < d) ++ld;
+  const int quad = (int)(n / (d / 4));
+  long long r = n - quad * (d / 4);
+  const bool swap = r > d / 8;
+  if (swap) r = d / 4 - r;
+  const unsigned long long pi61 = 0x6487ED5110B4611Aull;  // pi 2^61
+  const unsigned long long one = 1ull << 62;
+  const unsigned long long th = fx_mulhi(pi61, (unsigned long long)r << (66 - ld));  // 2 pi r / d, 62 fractional bits
+  const unsigned long long u = fx_mulhi(th << 1, th << 1);
+  unsigned long long vc = one, vs = one;
+#pragma unroll
+  for (int k = 18; k >= 2; k -= 2) {
+    vc = one - fx_mulhi(u << 1, vc << 1) / (unsigned long long)(k * (k - 1));
+    vs = one - fx_mulhi(u << 1, vs << 1) / (unsigned long long)(k * (k + 1));
+  }
+  vs = fx_mulhi(th << 1, vs << 1);
+  long long c = (long long)(swap ? vs : vc), s = (long long)(swap ? vc : vs);
+  // quadrant: multiply by i^quad
+  for (int i = 0; i < quad; ++i) {
+    const long long t = c;
+    c = -s;
+    s = t;
+  }
+  return {c, s};
+}
+
+// a value as two signed 32-bit digits (hi 2^32 + lo); lo = INT_MIN, which has
+// no negative, is moved by one unit
+struct FxDigits {
+  int h, l;
+};
+__host__ __device__ constexpr FxDigits fx_digits(long long v) {
+  int l = (int)(unsigned)(unsigned long long)v;
+  if (l == INT_MIN) {
+    v += 1;
+    l += 1;
+  }
+  return {(int)((v - l) >> 32), l};
+}
+// drop the last 62 - bits fractional bits, rounded
+__host__ __device__ constexpr long long fx_quant(long long v, int bits) {
+  return bits == 62 ? v : (v + (1ll << (61 - bits))) >> (62 - bits);
+}
+// exp(-2 pi i num/den) as a table entry
+__host__ __device__ inline fxw fx_twiddle(long num, long den) {
+  const FxRoot r = fx_root((int)(num % den), (int)den);
+  const FxDigits c = fx_digits(fx_quant(r.c, kFxTw)), s = fx_digits(fx_quant(-r.s, kFxTw));
+  fxw w;
+  w.x = c.h;
+  w.y = c.l;
+  w.z = s.h;
+  w.w = s.l;
+  return w;
+}
+// sin(pi j / N) / 2, j <= N/2, as a table entry with 62 fractional bits
+__host__ __device__ inline int2 fx_half_sine(int j, int N) {
+  const FxDigits s = fx_digits(fx_root(j, 2 * N).s >> 1);
+  int2 r;
+  r.x = s.h;
+  r.y = s.l;
+  return r;
+}
+
+// ---- arithmetic ----------------------------------------------------------------
+__host__ __device__ __forceinline__ int fx_lo(long long v) { return (int)(unsigned)(unsigned long long)v; }
+// high signed digit: v = fx_hi(v) 2^32 + fx_lo(v)
+__host__ __device__ __forceinline__ int fx_hi(long long v) {
+  return (int)(v >> 32) + (int)((unsigned)(unsigned long long)v >> 31);
+}
+__host__ __device__ __forceinline__ long long fx_wide(int a, int b) { return (long long)a * (long long)b; }
+
+// (acc 2^32 + low word of mid) >> s, s <= 32
+__host__ __device__ __forceinline__ long long fx_take(long long acc, long long mid, unsigned s) {
+#ifdef __CUDA_ARCH__
+  const unsigned m = (unsigned)mid, al = (unsigned)acc, ah = (unsigned)(acc >> 32);
+  const unsigned lo = __funnelshift_rc(m, al, s), hi = __funnelshift_rc(al, ah, s);
+  return (long long)(((unsigned long long)hi << 32) | lo);
+#else
+  const unsigned m = (unsigned)mid;
+  if (s == 32) return acc;
+  return (long long)(((unsigned long long)acc << (32 - s)) | (m >> s));
+#endif
+}
+
+// v * w for real v and a constant of F fractional bits (digits h, l), rounded.
+// The product of the two low digits (at most 2^(62-F) units) is left out.
+template <int F>
+__host__ __device__ __forceinline__ long long fx_rmul(long long v, int h, int l) {
+  const int vh = fx_hi(v), vl = fx_lo(v);
+  const long long mid = (1ll << (F - 33)) + fx_wide(vh, l) + fx_wide(vl, h);
+  return fx_take(fx_wide(vh, h) + (mid >> 32), mid, F - 32);
+}
+
+// w * v / 2^(32 + s), rounded; rnd = 2^(s-1)
+__host__ __device__ __forceinline__ fx2 fx_cmul(const fxw& w, fx2 v, unsigned s, long long rnd) {
+  const int xh = fx_hi(v.x), xl = fx_lo(v.x), yh = fx_hi(v.y), yl = fx_lo(v.y);
+  const int nh = -w.z, nl = -w.w;
+  const long long mr = rnd + fx_wide(xh, w.y) + fx_wide(xl, w.x) + fx_wide(yh, nl) + fx_wide(yl, nh);
+  const long long mi = rnd + fx_wide(xh, w.w) + fx_wide(xl, w.z) + fx_wide(yh, w.y) + fx_wide(yl, w.x);
+  fx2 r;
+  r.x = fx_take((mr >> 32) + fx_wide(xh, w.x) + fx_wide(yh, nh), mr, s);
+  r.y = fx_take((mi >> 32) + fx_wide(xh, w.z) + fx_wide(yh, w.x), mi, s);
+  return r;
+}
+
+// v / 2^sh, ties to even: a few bits are dropped, so ties are frequent, and
+// the prefix sum would add up the bias of rounding them one way
+__host__ __device__ __forceinline__ long long fx_shift(long long v, unsigned sh) {
+  const long long half = (1ll << sh) >> 1;
+  return (v + (sh ? half - 1 + ((v >> sh) & 1) : 0)) >> sh;
+}
+
+__host__ __device__ __forceinline__ fx2 fx_add(fx2 a, fx2 b) {
+  a.x += b.x;
+  a.y += b.y;
+  return a;
+}
+__host__ __device__ __forceinline__ fx2 fx_sub(fx2 a, fx2 b) {
+  a.x -= b.x;
+  a.y -= b.y;
+  return a;
+}
+
+// v * exp(-2 pi i K / R), the trivial and the diagonal roots without the
+// general product
+template <int K, int R>
+__host__ __device__ __forceinline__ fx2 fx_rotate(fx2 v) {
+  constexpr FxRoot root = fx_root(K, R);
+  fx2 r;
+  if constexpr (K == 0) {
+    r = v;
+  } else if constexpr (4 * K == R) {  // -i
+    r.x = v.y;
+    r.y = -v.x;
+  } else if constexpr (8 * K == R || 8 * K == 3 * R) {  // (+-1 - i) / sqrt 2
+    constexpr long long c63 = fx_root(1, 8).c << 1;
+    constexpr FxDigits c = fx_digits(c63);
+    const long long a = fx_rmul<63>(v.x + v.y, c.h, c.l), b = fx_rmul<63>(v.y - v.x, c.h, c.l);
+    if constexpr (8 * K == R) {
+      r.x = a;
+      r.y = b;
+    } else {
+      r.x = b;
+      r.y = -a;
+    }
+  } else {
+    constexpr FxDigits c = fx_digits(root.c), s = fx_digits(-root.s);
+    fxw w;
+    w.x = c.h;
+    w.y = c.l;
+    w.z = s.h;
+    w.w = s.l;
+    r = fx_cmul(w, v, 30, 1ll << 29);
+  }
+  return r;
+}
+
+template <int S, int K, int R>
+struct FxStage {  // butterflies of the radix-2 stage with half-length S, index K
+  static __host__ __device__ __forceinline__ void run(fx2 (&x)[R]) {
+#pragma unroll
+    for (int b = 0; b < R; b += 2 * S) {
+      const fx2 u = x[b + K], t = fx_rotate<K, 2 * S>(x[b + K + S]);
+      x[b + K] = fx_add(u, t);
+      x[b + K + S] = fx_sub(u, t);
+    }
+    if constexpr (K + 1 < S)
+      FxStage<S, K + 1, R>::run(x);
+    else if constexpr (2 * S < R)
+      FxStage<2 * S, 0, R>::run(x);
+  }
+};
+
+// in-register forward DFT of length R, natural order in and out
+template <int R>
+__host__ __device__ __forceinline__ void fx_dft(fx2 (&x)[R]) {
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    int j = 0;
+#pragma unroll
+    for (int b = 1; b < R; b <<= 1) j = (j << 1) | ((i & b) ? 1 : 0);
+    if (j > i) {
+      const fx2 t = x[i];
+      x[i] = x[j];
+      x[j] = t;
+    }
+  }
+  FxStage<1, 0, R>::run(x);
+}
+
+// ---- conversions -----------------------------------------------------------------
+__host__ __device__ __forceinline__ unsigned fx_dhi(double v) {
+#ifdef __CUDA_ARCH__
+  return (unsigned)__double2hiint(v);
+#else
+  unsigned long long b;
+  __builtin_memcpy(&b, &v, 8);
+  return (unsigned)(b >> 32);
+#endif
+}
+__host__ __device__ __forceinline__ unsigned fx_dlo(double v) {
+#ifdef __CUDA_ARCH__
+  return (unsigned)__double2loint(v);
+#else
+  unsigned long long b;
+  __builtin_memcpy(&b, &v, 8);
+  return (unsigned)b;
+#endif
+}
+
+// v as an integer multiple of 2^(E - 1022 - S1), truncated; E >= 1 is at least
+// v's exponent field.  mag: |result| >> 32.
+template <int S1>
+__host__ __device__ __forceinline__ long long fx_from_double(double v, int E, unsigned& mag) {
+  const unsigned hi = fx_dhi(v), lo = fx_dlo(v);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  const unsigned mh = (hi & 0xfffffu) | (e > 0 ? 0x100000u : 0u);  // subnormals have no leading one
+  int d = E - (e > 0 ? e : 1);
+  d = d > 63 ? 63 : d;
+  unsigned long long m = (((unsigned long long)mh << 32) | lo) << (S1 - 53);
+  m >>= d;
+  mag = (unsigned)(m >> 32);
+  return (hi >> 31) ? -(long long)m : (long long)m;
+}
+
+// d * 2^q for the few q at which the result could leave the normal range
+static __device__ __noinline__ double fx_scale_far(double d, int q) { return scalbn(d, q); }
+
+// v * 2^q.  The hardware conversion rounds to nearest (one FP64-pipe
+// operation); the exponent is added with integer instructions.  The far case
+// stays a call: inlined, its products would be issued on the FP64 pipe for
+// every value and discarded.
+__device__ __forceinline__ double fx_to_double(long long v, int q) {
+  const double d = __ll2double_rn(v);
+  if (q < -1000 || q > 900) return fx_scale_far(d, q);
+  const int hi = __double2hiint(d);
+  return __hiloint2double(v == 0 ? hi : hi + (q << 20), __double2loint(d));
+}
+
+// ---- shapes ----------------------------------------------------------------------
+// Radices per length and lanes per line.  The first radix is the largest (its
+// products round at the finest scale), and a lane holds N / TPL values; the
+// following radices are at most 8 where that keeps every shift <= kFxMaxShift
+// without giving up bits of S1.
+template <int N, int TPL> struct FixShape;
+template <> struct FixShape<32, 4> { enum { NP = 2, R0 = 8, R1 = 4, R2 = 1, R3 = 1 }; };
+template <> struct FixShape<64, 8> { enum { NP = 2, R0 = 8, R1 = 8, R2 = 1, R3 = 1 }; };
+template <> struct FixShape<128, 8> { enum { NP = 2, R0 = 16, R1 = 8, R2 = 1, R3 = 1 }; };
+template <> struct FixShape<256, 16> { enum { NP = 2, R0 = 16, R1 = 16, R2 = 1, R3 = 1 }; };
+template <> struct FixShape<512, 64> { enum { NP = 3, R0 = 8, R1 = 8, R2 = 8, R3 = 1 }; };
+template <> struct FixShape<512, 128> { enum { NP = 4, R0 = 8, R1 = 4, R2 = 4, R3 = 4 }; };
+template <> struct FixShape<1024, 64> { enum { NP = 3, R0 = 16, R1 = 8, R2 = 8, R3 = 1 }; };
+template <> struct FixShape<1024, 128> { enum { NP = 4, R0 = 8, R1 = 8, R2 = 4, R3 = 4 }; };
+template <> struct FixShape<2048, 256> { enum { NP = 4, R0 = 8, R1 = 8, R2 = 8, R3 = 4 }; };
+template <> struct FixShape<4096, 256> { enum { NP = 3, R0 = 16, R1 = 16, R2 = 16, R3 = 1 }; };
+template <> struct FixShape<8192, 512> { enum { NP = 4, R0 = 16, R1 = 8, R2 = 8, R3 = 8 }; };
+
+__host__ __device__ constexpr int fx_log2(int v) {
+  int l = 0;
+  while ((1 << l) < v) ++l;
+  return l;
+}
+
+// the scale plan of a shape: S1 and the shifts
+template <int R0, int R1, int R2, int R3>
+struct FixScale {
+  enum {
+    W0 = fx_log2(R0), W1 = fx_log2(R1), W2 = fx_log2(R2), W3 = fx_log2(R3),
+    // bits by which a radix above 8 would exceed kFxMaxShift, taken from S1
+    X = (W1 > 3 ? W1 - 3 : 0) + (W2 > 3 ? W2 - 3 : 0) + (W3 > 3 ? W3 - 3 : 0),
+    S1 = 61 - W0 - X
+  };
+  // right shift, in all, of the values that enter pass p = 1 .. NP-1 (and are
+  // twiddled there); 2^lb bounds the line's sum of |re| + |im| at the scale of
+  // S1.  A pass shifts by at most kFxMaxShift, so a pass before the last takes
+  // more than its own bound asks for where the later ones could not.
+  template <int NP>
+  static __host__ __device__ __forceinline__ int shift_at(int p, int lb) {
+    int all = S1 + 1 + W0 + W1 + W2 + W3, own = S1 + 1 + W0 + W1 + (p >= 2 ? W2 : 0) + (p >= 3 ? W3 : 0);
+    all = (all < lb ? all : lb) - 62;
+    own = (own < lb ? own : lb) - 62;
+    const int rest = all - kFxMaxShift * (NP - 1 - p);
+    own = own > rest ? own : rest;
+    return own > 0 ? own : 0;
+  }
+};
+
+// entries of the pass tables [q][k] = w_{Ls r}^{q k}, passes 2 .. NP
+template <typename S>
+__host__ __device__ constexpr int fix_tp_entries() {
+  return (int)S::R0 * S::R1 + (S::NP > 2 ? (int)S::R0 * S::R1 * S::R2 : 0) +
+         (S::NP > 3 ? (int)S::R0 * S::R1 * S::R2 * S::R3 : 0);
+}
+
+// padded position of line element i: one slot per 8, so that lanes 8 elements
+// apart (the first pass's stores, the chunks of the scan) hit distinct banks
+__host__ __device__ constexpr int fpad(int i) { return i + (i >> 3); }
+// fpad(base + q step), the step's part folded into a constant where it is a multiple of 8
+template <int STEP>
+__host__ __device__ __forceinline__ int fpad_step(int base, int q) {
+  return STEP % 8 == 0 ? fpad(base) + q * (STEP + STEP / 8) : fpad(base + q * STEP);
+}
+
+// ---- one line in shared memory ------------------------------------------------------
+__device__ __forceinline__ void fx_line_sync(int tpl) {
+  if (tpl <= 32) {
+    __syncwarp();
+  } else if (tpl >= 256) {
+    __syncthreads();
+  } else {  // the lanes of one line only; barrier 0 is the CTA's
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)(threadIdx.x / tpl)), "r"(tpl) : "memory");
+  }
+}
+
+// identity epilogue of FixLine::run
+struct FixNoPost {
+  __device__ __forceinline__ void start() {}
+  __device__ __forceinline__ double2 operator()(int, double2 v) { return v; }
+};
+
+template <int N, int TPL>
+struct FixLine {
+  typedef FixShape<N, TPL> S;
+  typedef FixScale<S::R0, S::R1, S::R2, S::R3> SC;
+  enum { NL = N / TPL, H = N / 2, CH = H / TPL, NW = TPL / 32, S1 = SC::S1,
+         // bits dropped from the magnitudes' high words so that their sum over
+         // the line fits in 32 bits
+         G = (S1 - 32) + fx_log2(2 * N) - 31 > 0 ? (S1 - 32) + fx_log2(2 * N) - 31 : 0 };
+  // largest value over the line's lanes; slot: NW words of scratch
+  static __device__ __forceinline__ unsigned line_max(unsigned v, unsigned* slot, int t) {
+    if constexpr (TPL >= 32) {
+      v = __reduce_max_sync(0xffffffffu, v);
+    } else {
+#pragma unroll
+      for (int d = 1; d < TPL; d <<= 1) {
+        const unsigned o = __shfl_xor_sync(0xffffffffu, v, d, TPL);
+        v = v > o ? v : o;
+      }
+    }
+    if constexpr (TPL > 32) {
+      if ((t & 31) == 0) slot[t >> 5] = v;
+      fx_line_sync(TPL);
+#pragma unroll
+      for (int w = 0; w < NW; ++w) v = v > slot[w] ? v : slot[w];
+    } else {
+      __syncwarp();
+    }
+    return v;
+  }
+
+  template <int R, int LSP, bool FIRST>
+  static __device__ __forceinline__ void pass(fx2* a, int t, const fxw* tp, int sh) {
+    constexpr int GR = N / R, PER = (GR + TPL - 1) / TPL;
+    const bool active = GR >= TPL || t < GR;  // a radix above N / TPL leaves lanes idle in its pass
+    fx2 x[PER][R];
+    const unsigned s = (unsigned)(kFxTw - 32 + sh);
+    const long long rnd = 1ll << (s - 1);
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      if (!active) break;
+      const int l = t + TPL * i, k = l & (LSP - 1);
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        fx2 v = a[fpad_step<GR>(l, q)];
+        if constexpr (!FIRST) {
+          if (q > 0) {
+            // exact roots (k = 0) leave ties: rounded up and down in turn
+            v = fx_cmul(tp[q * LSP + k], v, s, rnd - (q & 1));
+          } else {
+            v.x = fx_shift(v.x, sh);
+            v.y = fx_shift(v.y, sh);
+          }
+        }
+        x[i][q] = v;
+      }
+      fx_dft<R>(x[i]);
+    }
+    fx_line_sync(TPL);
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      if (!active) break;
+      const int l = t + TPL * i, j = l / LSP, k = l & (LSP - 1);
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+        a[LSP == 1 && R % 8 == 0 ? fpad(j * R) + fpad(q) : fpad_step<LSP>(j * LSP * R + k, q)] = x[i][q];
+    }
+    fx_line_sync(TPL);
+  }
+
+  // Unnormalised DST-I of the line (doubles at fpad(1) .. fpad(N-1)) in place.
+  // scr: 2 max(NW, 4) 16-byte slots of the line.  post(m, value) is applied to
+  // every result before it is stored (post.start() earlier, for its loads).
+  // Every lane of the line must call it, and the line's input must be visible
+  // to them.
+  template <typename POST>
+  static __device__ __forceinline__ void run(double2* line, int t, const int2* hs, const fxw* tp, void* scr,
+                                             POST& post) {
+    fx2* a = (fx2*)line;
+    fx2* s_scan = (fx2*)scr;
+    unsigned* s_max = (unsigned*)((char*)scr + 16 * NW);
+    unsigned* s_sum = s_max + NW;
+    int E;
+    bool nonfinite;
+    {  // ---- scale, pre-twiddle: the lane's pairs (m, N - m), m = 1 + t + TPL i
+      double2 za[NL / 2], zb[NL / 2];
+      unsigned mx = 0;
+#pragma unroll
+      for (int i = 0; i < NL / 2; ++i) {
+        za[i] = line[fpad_step<TPL>(1 + t, i)];
+        zb[i] = line[fpad_step<TPL>(N - 1 - t, -i)];
+        const unsigned h0 = fx_dhi(za[i].x) & 0x7fffffffu, h1 = fx_dhi(za[i].y) & 0x7fffffffu;
+        const unsigned h2 = fx_dhi(zb[i].x) & 0x7fffffffu, h3 = fx_dhi(zb[i].y) & 0x7fffffffu;
+        mx = max(mx, max(max(h0, h1), max(h2, h3)));
+      }
+      mx = line_max(mx, s_max, t);
+      E = (int)(mx >> 20);
+      nonfinite = E == 0x7ff;
+      E = E > 1 ? E : 1;
+      unsigned sum = 0;
+#pragma unroll
+      for (int i = 0; i < NL / 2; ++i) {
+        unsigned g0, g1, g2, g3;
+        const fx2 u = {fx_from_double<S1>(za[i].x, E, g0), fx_from_double<S1>(za[i].y, E, g1)};
+        const fx2 v = {fx_from_double<S1>(zb[i].x, E, g2), fx_from_double<S1>(zb[i].y, E, g3)};
+        sum += ((g0 >> G) + (g1 >> G)) + ((g2 >> G) + (g3 >> G));
+        const int2 h = hs[1 + t + TPL * i];
+        const fx2 p = fx_add(u, v), d = fx_sub(u, v);
+        const fx2 A = {fx_rmul<62>(p.x, h.x, h.y), fx_rmul<62>(p.y, h.x, h.y)};
+        // the quarter, ties rounded up and down in turn
+        const fx2 B = {(d.x + 1 + (i & 1)) >> 2, (d.y + 1 + (i & 1)) >> 2};
+        a[fpad_step<TPL>(1 + t, i)] = fx_add(A, B);
+        a[fpad_step<TPL>(N - 1 - t, -i)] = fx_sub(A, B);  // m = N/2: its own partner, B = 0
+      }
+      if (t == 0) a[0] = {0, 0};
+      if constexpr (TPL >= 32) {
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if constexpr (TPL > 32) {
+          if ((t & 31) == 0) s_sum[t >> 5] = sum;
+        }
+      } else {
+#pragma unroll
+        for (int d = 1; d < TPL; d <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d, TPL);
+      }
+      fx_line_sync(TPL);
+      pass<S::R0, 1, true>(a, t, tp, 0);
+      if constexpr (TPL > 32) {
+        sum = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) sum += s_sum[w];
+      }
+      sum += 2 * N;
+      const int lb = 32 + G + 32 - __clz(sum);
+      int t1 = 0, tn = 0;
+      tn = SC::template shift_at<S::NP>(1, lb);
+      pass<S::R1, S::R0, false>(a, t, tp, tn);
+      if constexpr (S::NP > 2) {
+        t1 = tn;
+        tn = SC::template shift_at<S::NP>(2, lb);
+        pass<S::R2, S::R0 * S::R1, false>(a, t, tp + S::R0 * S::R1, tn - t1);
+      }
+      if constexpr (S::NP > 3) {
+        t1 = tn;
+        tn = SC::template shift_at<S::NP>(3, lb);
+        pass<S::R3, S::R0 * S::R1 * S::R2, false>(a, t, tp + S::R0 * S::R1 + S::R0 * S::R1 * S::R2, tn - t1);
+      }
+      E += tn;
+    }
+    post.start();
+    // ---- split into C_k and S_k and prefix sum of C: the lane's chunk k = CH t + i
+    const int q = E - 1022 - S1;  // results are multiples of 2^q
+    fx2 cc[CH], ss[CH];
+    fx2 tot = {0, 0};
+#pragma unroll
+    for (int i = 0; i < CH; ++i) {
+      const int k = CH * t + i;
+      const fx2 Yk = a[fpad(k)];
+      fx2 Ym = {0, 0};
+      if (i > 0 || t > 0) Ym = a[fpad(N - k)];
+      tot = fx_add(tot, fx_add(Yk, Ym));
+      cc[i] = tot;
+      ss[i].x = Ym.y - Yk.y;
+      ss[i].y = Yk.x - Ym.x;
+    }
+    fx2 inc = tot;
+    const int lw = t & 31;
+    constexpr int SW = TPL < 32 ? TPL : 32;
+#pragma unroll
+    for (int d = 1; d < SW; d <<= 1) {
+      const long long ux = __shfl_up_sync(0xffffffffu, inc.x, d, SW), uy = __shfl_up_sync(0xffffffffu, inc.y, d, SW);
+      if ((lw & (SW - 1)) >= d) {
+        inc.x += ux;
+        inc.y += uy;
+      }
+    }
+    if constexpr (TPL > 32) {
+      if (lw == 31) s_scan[t >> 5] = inc;
+    }
+    fx_line_sync(TPL);  // also: every read of Y precedes the stores below
+    if constexpr (TPL > 32) {
+      for (int w = 0; w < (t >> 5); ++w) inc = fx_add(inc, s_scan[w]);
+    }
+    const fx2 before = fx_sub(inc, tot);
+    const double bad = __longlong_as_double(0x7ff8000000000000ll);
+#pragma unroll
+    for (int i = 0; i < CH; ++i) {
+      const int k = CH * t + i;
+      const fx2 o = fx_add(before, cc[i]);
+      double2 vo = make_double2(fx_to_double(o.x, q), fx_to_double(o.y, q));
+      double2 ve = make_double2(fx_to_double(ss[i].x, q), fx_to_double(ss[i].y, q));
+      if (nonfinite) vo = ve = make_double2(bad, bad);
+      if (i > 0 || t > 0) line[fpad(2 * k)] = post(2 * k, ve);
+      line[fpad(2 * k + 1)] = post(2 * k + 1, vo);
+    }
+    fx_line_sync(TPL);
+  }
+};
+
+// lines of N <= 16 points: the whole line in one lane's registers
+template <int N>
+struct FixLine<N, 1> {
+  enum { S1 = 61 - fx_log2(N) };
+  template <typename POST>
+  static __device__ __forceinline__ void run(double2* line, int, const int2* hs, const fxw*, void*, POST& post) {
+    unsigned mx = 0;
+#pragma unroll
+    for (int j = 1; j < N; ++j) {
+      const double2 z = line[fpad(j)];
+      mx = max(mx, max(fx_dhi(z.x) & 0x7fffffffu, fx_dhi(z.y) & 0x7fffffffu));
+    }
+    int E = (int)(mx >> 20);
+    const bool nonfinite = E == 0x7ff;
+    E = E > 1 ? E : 1;
+    fx2 x[N];
+    x[0] = {0, 0};
+#pragma unroll
+    for (int j = 1; j <= N / 2; ++j) {
+      unsigned g;
+      const double2 za = line[fpad(j)], zb = line[fpad(N - j)];
+      const fx2 u = {fx_from_double<S1>(za.x, E, g), fx_from_double<S1>(za.y, E, g)};
+      const fx2 v = {fx_from_double<S1>(zb.x, E, g), fx_from_double<S1>(zb.y, E, g)};
+      if (j == N / 2) {
+        x[j] = u;
+      } else {
+        const int2 h = hs[j];
+        const fx2 p = fx_add(u, v), d = fx_sub(u, v);
+        const fx2 A = {fx_rmul<62>(p.x, h.x, h.y), fx_rmul<62>(p.y, h.x, h.y)};
+        const fx2 B = {(d.x + 1 + (j & 1)) >> 2, (d.y + 1 + (j & 1)) >> 2};
+        x[j] = fx_add(A, B);
+        x[N - j] = fx_sub(A, B);
+      }
+    }
+    fx_dft<N>(x);
+    post.start();
+    const int q = E - 1022 - S1;
+    const double bad = __longlong_as_double(0x7ff8000000000000ll);
+    fx2 sum = x[0];
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) {
+      if (k > 0) {
+        const fx2 Yk = x[k], Ym = x[N - k];
+        sum = fx_add(sum, fx_add(Yk, Ym));
+        double2 ve = make_double2(fx_to_double(Ym.y - Yk.y, q), fx_to_double(Yk.x - Ym.x, q));
+        if (nonfinite) ve = make_double2(bad, bad);
+        line[fpad(2 * k)] = post(2 * k, ve);
+      }
+      double2 vo = make_double2(fx_to_double(sum.x, q), fx_to_double(sum.y, q));
+      if (nonfinite) vo = make_double2(bad, bad);
+      line[fpad(2 * k + 1)] = post(2 * k + 1, vo);
+    }
+  }
+};
+
+// line stride in 16-byte slots: odd for short lines (one line per lane, or
+// tiles of 8 and more columns), 2 mod 8 for long ones (tiles of 4 columns), so
+// that column-wise tile copies spread over the banks
+template <int N>
+__host__ __device__ constexpr int fix_line_stride() {
+  return N <= 256 ? fpad(N) | 1 : ((fpad(N) + 7) / 8) * 8 + 2;
+}
+
+// pass-table entries of (N, TPL); 0 when the line stays in one lane
+template <int N, int TPL>
+__host__ __device__ constexpr int fix_table_entries() {
+  if constexpr (TPL == 1)
+    return 0;
+  else
+    return fix_tp_entries<FixShape<N, TPL>>();
+}
+
+// Pass table of the radices r[0 .. np-1], host or device: entry e of pass p is
+// w_{Ls r_p}^{q k}, e = q Ls + k.
+struct FixRadices {
+  int np, r[4];
+};
+__host__ __device__ inline fxw fix_table_entry(const FixRadices& f, int e) {
+  int ls = f.r[0];
+  for (int p = 1; p < f.np; ++p) {
+    const int n = ls * f.r[p];
+    if (e < n) return fx_twiddle((long)(e / ls) * (e % ls), n);
+    e -= n;
+    ls = n;
+  }
+  return fxw{0, 0, 0, 0};
+}
+template <int N, int TPL>
+__host__ __device__ constexpr FixRadices fix_radices() {
+  typedef FixShape<N, TPL> S;
+  return {S::NP, {S::R0, S::R1, S::R2, S::R3}};
+}
+
+}  // namespace csl

@@ -1,6 +1,7 @@
-// Launch wrappers of the sine-transform passes for one real type CSL_T
-// (instantiated by csl_pass64.cu and csl_pass32.cu so that the two
-// precisions compile in parallel).
+// Launch wrappers of the sine-transform passes for one real type and one
+// length (launch_*_n), and, where CSL_T is defined, the dispatch over the
+// lengths.  csl_pass32.cu holds every FP32 length; the FP64 ones are spread
+// over csl_pass64*.cu so that they compile in parallel.
 #pragma once
 #include "csl_passes.cuh"
 
@@ -35,24 +36,6 @@ cudaError_t launch_row_n(int load, int store, const RowArgs<T>& a, const PassLau
   return cudaErrorInvalidValue;
 }
 
-template <typename T>
-cudaError_t launch_row(int N, int wide, int load, int store, const RowArgs<T>& a, const PassLaunch& L,
-                       cudaStream_t s, const RowArgs<T>* batch, int nsys) {
-  if (pass_is_big(N)) return launch_row_big<T>(N, load, store, a, L, s, batch, nsys);
-  switch (N) {
-#define CASE(NN)                                                                    \
-  case NN:                                                                          \
-    if constexpr (NN >= 512) {                                                      \
-      if (wide == 1) return launch_row_n<T, NN, 1>(load, store, a, L, s, batch, nsys); \
-      if (wide == 2) return launch_row_n<T, NN, 2>(load, store, a, L, s, batch, nsys); \
-    }                                                                               \
-    return launch_row_n<T, NN, 0>(load, store, a, L, s, batch, nsys);
-    CSL_FOR_EACH_N(CASE)
-#undef CASE
-  }
-  return cudaErrorInvalidValue;
-}
-
 template <typename T, int N, int W>
 cudaError_t launch_strided_n(bool mid, const StridedArgs<T>& a, const PassLaunch& L, cudaStream_t s,
                              const StridedArgs<T>* batch, int nsys) {
@@ -61,61 +44,31 @@ cudaError_t launch_strided_n(bool mid, const StridedArgs<T>& a, const PassLaunch
   return launch_k(L.pdl != 0, k_strided<T, N, W, false>, grid, L.threads, L.smem, s, a, batch, L.blocks);
 }
 
-template <typename T>
-cudaError_t launch_strided(int N, int wide, bool mid, const StridedArgs<T>& a, const PassLaunch& L,
-                           cudaStream_t s, const StridedArgs<T>* batch, int nsys) {
-  if constexpr (sizeof(T) == 4) {
-    if (L.tc) return launch_strided_tc(N, L.tc, mid, a, L, s, batch, nsys);
-  }
-  if (pass_is_big(N)) return launch_strided_big<T>(N, mid, a, L, s, batch, nsys);
-  switch (N) {
-#define CASE(NN)                                                                  \
-  case NN:                                                                        \
-    if constexpr (NN >= 512) {                                                    \
-      if (wide == 1) return launch_strided_n<T, NN, 1>(mid, a, L, s, batch, nsys); \
-      if (wide == 2) return launch_strided_n<T, NN, 2>(mid, a, L, s, batch, nsys); \
-    }                                                                             \
-    return launch_strided_n<T, NN, 0>(mid, a, L, s, batch, nsys);
-    CSL_FOR_EACH_N(CASE)
-#undef CASE
-  }
-  return cudaErrorInvalidValue;
-}
-
-template <typename T>
-cudaError_t set_pass_attrs() {
+template <typename T, int N, int W>
+cudaError_t set_pass_attrs_n() {
   cudaError_t e = cudaSuccess;
-#define SETA(k) \
-  if (e == cudaSuccess) e = allow_dyn_smem((const void*)k);
-#define VARIANT(NN, W)                                 \
-  SETA((k_row<T, NN, W, LOAD_V, STORE_T>))             \
-  SETA((k_row<T, NN, W, LOAD_LANCZOS, STORE_T>))       \
-  SETA((k_row<T, NN, W, LOAD_T, STORE_Z>))             \
-  SETA((k_row<T, NN, W, LOAD_T, STORE_Z_UPDATE>))      \
-  SETA((k_row<T, NN, W, LOAD_T, STORE_D>))             \
-  SETA((k_strided<T, NN, W, true>))                    \
-  SETA((k_strided<T, NN, W, false>))                   \
-  if constexpr (sizeof(T) == 4) {                      \
-    SETA((k_row<T, NN, W, LOAD_LANCZOS_V64, STORE_T>)) \
-    SETA((k_row<T, NN, W, LOAD_T, STORE_Z_UPDATE_V64>)) \
+#define SETA(...) \
+  if (e == cudaSuccess) e = allow_dyn_smem((const void*)__VA_ARGS__);
+  SETA(k_row<T, N, W, LOAD_V, STORE_T>)
+  SETA(k_row<T, N, W, LOAD_LANCZOS, STORE_T>)
+  SETA(k_row<T, N, W, LOAD_T, STORE_Z>)
+  SETA(k_row<T, N, W, LOAD_T, STORE_Z_UPDATE>)
+  SETA(k_row<T, N, W, LOAD_T, STORE_D>)
+  SETA(k_strided<T, N, W, true>)
+  SETA(k_strided<T, N, W, false>)
+  if constexpr (sizeof(T) == 4) {
+    SETA(k_row<T, N, W, LOAD_LANCZOS_V64, STORE_T>)
+    SETA(k_row<T, N, W, LOAD_T, STORE_Z_UPDATE_V64>)
   }
-#define CASE(NN) VARIANT(NN, 0)
-  CSL_FOR_EACH_N(CASE)
-#undef CASE
-  VARIANT(512, 1)
-  VARIANT(1024, 1)
-  VARIANT(512, 2)
-  VARIANT(1024, 2)
-#undef VARIANT
 #undef SETA
-  if (e == cudaSuccess) e = set_pass_attrs_big<T>();
   return e;
 }
 
-template cudaError_t launch_row<CSL_T>(int, int, int, int, const RowArgs<CSL_T>&, const PassLaunch&,
-                                       cudaStream_t, const RowArgs<CSL_T>*, int);
-template cudaError_t launch_strided<CSL_T>(int, int, bool, const StridedArgs<CSL_T>&, const PassLaunch&,
-                                           cudaStream_t, const StridedArgs<CSL_T>*, int);
-template cudaError_t set_pass_attrs<CSL_T>();
+#define CSL_INSTANTIATE_PASS(T, N, W)                                                                            \
+  template cudaError_t launch_row_n<T, N, W>(int, int, const RowArgs<T>&, const PassLaunch&, cudaStream_t,       \
+                                             const RowArgs<T>*, int);                                            \
+  template cudaError_t launch_strided_n<T, N, W>(bool, const StridedArgs<T>&, const PassLaunch&, cudaStream_t,   \
+                                                 const StridedArgs<T>*, int);                                    \
+  template cudaError_t set_pass_attrs_n<T, N, W>();
 
 }  // namespace csl

@@ -19,9 +19,9 @@
 
 #include <vector>
 
-// FP32 passes: two CTAs of 256 threads per SM (at most 128 registers per
-// thread); the FP64 lines need the full register file
-#define CSL_PASS_MINB(T, V) (sizeof(T) == 4 && (V) < 3 ? ((V) == 2 ? 3 : 2) : 1)
+// two CTAs of 256 threads per SM (at most 128 registers per thread), three
+// with 128 lanes per line in FP32; one of a long line's
+#define CSL_PASS_MINB(T, V) ((V) < 3 ? (sizeof(T) == 4 && (V) == 2 ? 3 : 2) : 1)
 // The warp-per-line row passes of length 1024 that stream MINRES vectors
 // from HBM (the Lanczos step before the forward transform, the w/x update
 // after the inverse one) keep many loads in flight per lane, so they take the
@@ -45,7 +45,7 @@ struct RowArgs {
   int n, nrows;
   const typename C2<T>::t* tw;
   const T* hs;
-  const typename C2<T>::t* tp;    // extra twiddle table (LineDst::TP entries)
+  const typename C2<T>::t* tp;    // extra twiddle table (pass_tp_offset)
   const double2* vin;             // LOAD_V
   const typename C2<T>::t* tin;   // LOAD_T
   double2* vnew;                  // LOAD_LANCZOS: u' in, v_{j+1} out
@@ -80,26 +80,11 @@ struct StridedArgs {
   const void* sine_tc; // tensor-core variant: split-bf16 sine matrix in B-operand layout
 };
 
-// byte offsets of the shared-memory regions: twiddles | half sines | extra
-// twiddles | scan scratch (2 per line) | lines
-// (long lines, variant 3, read their tables from global memory)
-template <typename T, int N, int WIDE>
-__host__ __device__ constexpr size_t pass_tables_bytes() {
-  return LineDst<T, N, WIDE>::GLOBAL_TABLES
-             ? 0
-             : (size_t)(N / 2) * sizeof(typename C2<T>::t) + (((size_t)(N / 2 + 1) * sizeof(T) + 15) / 16) * 16 +
-                   (size_t)line_tp_size(N, WIDE) * sizeof(typename C2<T>::t);
-}
-// scan scratch per line: one complex per warp of the line (at least 4; the
-// long-line variant scans in FP64, so twice as many T-complex slots)
-template <typename T, int N, int WIDE>
-__host__ __device__ constexpr int pass_scratch() {
-  return (LineDst<T, N, WIDE>::TPL / 32 > 4 ? LineDst<T, N, WIDE>::TPL / 32 : 4) * (WIDE == 3 ? 2 : 1);
-}
+// shared-memory regions: tables | scan scratch (per line) | lines
 template <typename T, int N, int WIDE>
 __host__ __device__ constexpr size_t pass_smem_bytes(int lines) {
-  return pass_tables_bytes<T, N, WIDE>() + (size_t)lines * pass_scratch<T, N, WIDE>() * sizeof(typename C2<T>::t) +
-         (size_t)lines * LineDst<T, N, WIDE>::LS * sizeof(typename C2<T>::t);
+  typedef LineDst<T, N, WIDE> D;
+  return D::Tables::kBytes + (size_t)lines * (D::SCRATCH + D::LS) * sizeof(typename C2<T>::t);
 }
 // CTA size bound of the pass kernels: 256, or one long line's lanes
 template <int N, int WIDE>
@@ -134,21 +119,10 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_ROW_MINB(T, N
   constexpr int UBMAX = STORE == STORE_Z_UPDATE ? (wide_batch ? 4 : 2) : LOAD == LOAD_LANCZOS ? (wide_batch ? 16 : 4) : 8;
   constexpr int UB = NL < UBMAX ? NL : UBMAX;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  c_t* w_tw = (c_t*)smem_raw;
-  T* w_hs = (T*)(smem_raw + (size_t)(N / 2) * sizeof(c_t));
-  c_t* w_tp = (c_t*)(smem_raw + (size_t)(N / 2) * sizeof(c_t) + (((size_t)(N / 2 + 1) * sizeof(T) + 15) / 16) * 16);
-  const c_t* s_tw = w_tw;
-  const T* s_hs = w_hs;
-  const c_t* s_tp = w_tp;
   const int nlines = blockDim.x / TPL;
-  c_t* s_scr = (c_t*)(smem_raw + pass_tables_bytes<T, N, WIDE>());
-  c_t* lines = s_scr + pass_scratch<T, N, WIDE>() * nlines;
-  if constexpr (D::GLOBAL_TABLES) {
-    s_tw = a.tw;
-    s_hs = a.hs;
-  } else {
-    load_tables<T>(w_tw, w_hs, w_tp, a.tw, a.hs, a.tp, N, D::TP);  // constant: may overlap the predecessor
-  }
+  c_t* s_scr = (c_t*)(smem_raw + D::Tables::kBytes);
+  c_t* lines = s_scr + D::SCRATCH * nlines;
+  const auto tb = D::Tables::load(smem_raw, a.tw, a.hs, a.tp);  // constant: may overlap the predecessor
   pdl_wait();
   if (a.st && a.st->done) return;
   double lz = 0.0, wb = 0.0, wc = 0.0, xc = 0.0;
@@ -268,7 +242,7 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_ROW_MINB(T, N
       }
     }
     D::line_sync();
-    D::template run<false>(line, t, s_tw, s_hs, s_tp, s_scr);
+    D::template run<false>(line, t, tb, s_scr);
     if (valid) {
 #pragma unroll
       for (int i0 = 0; i0 < NL; i0 += UB) {
@@ -368,6 +342,23 @@ __device__ void mid_scalar_tail(const StridedArgs<T>& a, double g2acc, int bid, 
   store_scalar_fields(a.st, q);
 }
 
+// FP64 epilogue of the transforms in the MID pass; after the forward one mode m times its
+// scale s_m, and s_m |F|^2 into the Parseval sum
+struct MidScale {
+  const double* stab;  // the column's scales, mode m at (m - 1) stride
+  long stride;
+  bool valid, forward;
+  double part;
+  __device__ __forceinline__ void start() {}
+  __device__ __forceinline__ double2 operator()(int m, double2 F) {
+    if (!forward) return F;  // the inverse transform's results
+    const double sc = valid ? stab[(long)(m - 1) * stride] : 0.0;
+    const double2 v = make_double2(F.x * sc, F.y * sc);
+    part = fma(v.x, F.x, fma(v.y, F.y, part));
+    return v;
+  }
+};
+
 template <typename T, int N, int WIDE, bool MID>
 __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_PASS_MINB(T, WIDE)) k_strided(StridedArgs<T> a0, const StridedArgs<T>* batch, int bps) {
   typedef typename C2<T>::t c_t;
@@ -380,21 +371,10 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_PASS_MINB(T, 
   constexpr int NL = (N + TPL - 1) / TPL;
   constexpr int UB = NL < 8 ? NL : 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  c_t* w_tw = (c_t*)smem_raw;
-  T* w_hs = (T*)(smem_raw + (size_t)(N / 2) * sizeof(c_t));
-  c_t* w_tp = (c_t*)(smem_raw + (size_t)(N / 2) * sizeof(c_t) + (((size_t)(N / 2 + 1) * sizeof(T) + 15) / 16) * 16);
-  const c_t* s_tw = w_tw;
-  const T* s_hs = w_hs;
-  const c_t* s_tp = w_tp;
   const int C = blockDim.x / TPL;  // lines (columns) per tile, a power of two
-  c_t* s_scr = (c_t*)(smem_raw + pass_tables_bytes<T, N, WIDE>());
-  c_t* lines = s_scr + pass_scratch<T, N, WIDE>() * C;
-  if constexpr (D::GLOBAL_TABLES) {
-    s_tw = a.tw;
-    s_hs = a.hs;
-  } else {
-    load_tables<T>(w_tw, w_hs, w_tp, a.tw, a.hs, a.tp, N, D::TP);  // constant: may overlap the predecessor
-  }
+  c_t* s_scr = (c_t*)(smem_raw + D::Tables::kBytes);
+  c_t* lines = s_scr + D::SCRATCH * C;
+  const auto tb = D::Tables::load(smem_raw, a.tw, a.hs, a.tp);  // constant: may overlap the predecessor
   pdl_wait();
   if (a.st && a.st->done) return;
   __shared__ DevState s_pre;
@@ -433,51 +413,51 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_PASS_MINB(T, 
     cp_async_commit();
     cp_async_wait<0>();
     __syncthreads();
-    D::template run<false>(line, t, s_tw, s_hs, s_tp, s_scr);
+    if constexpr (MID && sizeof(T) == 8) {
+      // the scale and the Parseval sum are applied to the results while they
+      // are in registers
+      MidScale post = {a.stab + base + myl, a.line_stride, myl < Ch, true, 0.0};
+#pragma unroll 1
+      for (int pass = 0; pass < 2; ++pass) {  // one copy of the transform's code: two miss the instruction cache
+        D::run_post(line, t, tb, s_scr, post);
+        post.forward = false;
+      }
+      g2acc += post.part;
+    } else {
+    D::template run<false>(line, t, tb, s_scr);
     if (MID) {
       if (myl < Ch) {
         const int ix = col0 + myl;
         T murest = a.mu_col ? a.mu_col[ix] : (T)0;
         if (a.mu_outer) murest += a.mu_outer[o];
         T part = (T)0;
-        if (a.stab) {
-          for (int m = 1 + t; m <= n; m += TPL) {
+        // the lane's eigenvalues mu_m are loaded together before the
+        // scaling, so their latencies overlap instead of adding up
+        T mu[NL];
+#pragma unroll
+        for (int k = 0; k < NL; ++k) {
+          const int m = 1 + t + TPL * k;
+          mu[k] = m <= n ? a.mu_line[m - 1] : (T)0;
+        }
+#pragma unroll
+        for (int k = 0; k < NL; ++k) {
+          const int m = 1 + t + TPL * k;
+          if (m <= n) {
             const int pos = D::out_pos(m);
             c_t F = line[pos];
-            const T sc = (T)a.stab[base + (long)(m - 1) * a.line_stride + myl];
+            const T e = fma(a.gamma, murest + mu[k], a.alpha);
+            const T sc = a.cnorm * rsq(fma(e, e, a.beta2));
             part = fma(sc, fma(F.x, F.x, F.y * F.y), part);
             F.x *= sc;
             F.y *= sc;
             line[pos] = F;
           }
-        } else {
-          // the lane's eigenvalues mu_m are loaded together before the
-          // scaling, so their latencies overlap instead of adding up
-          T mu[NL];
-#pragma unroll
-          for (int k = 0; k < NL; ++k) {
-            const int m = 1 + t + TPL * k;
-            mu[k] = m <= n ? a.mu_line[m - 1] : (T)0;
-          }
-#pragma unroll
-          for (int k = 0; k < NL; ++k) {
-            const int m = 1 + t + TPL * k;
-            if (m <= n) {
-              const int pos = D::out_pos(m);
-              c_t F = line[pos];
-              const T e = fma(a.gamma, murest + mu[k], a.alpha);
-              const T sc = a.cnorm * rsq(fma(e, e, a.beta2));
-              part = fma(sc, fma(F.x, F.x, F.y * F.y), part);
-              F.x *= sc;
-              F.y *= sc;
-              line[pos] = F;
-            }
-          }
         }
         g2acc += (double)part;
       }
       D::line_sync();
-      D::template run<true>(line, t, s_tw, s_hs, s_tp, s_scr);
+      D::template run<true>(line, t, tb, s_scr);
+    }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < C * n; i += blockDim.x) {
@@ -505,6 +485,9 @@ struct PassLaunch {
 // per line: wide = 0, 1, 2); the autotuner picks one per pass.
 inline bool pass_has_wide(int N) { return N == 512 || N == 1024; }
 inline int pass_num_variants(int N) { return pass_has_wide(N) ? 3 : 1; }
+// the first variant the tuner tries: the FP64 form's variant 0 is its 1
+template <typename T>
+inline int pass_first_variant(int N) { return sizeof(T) == 8 && pass_has_wide(N) ? 1 : 0; }
 
 // Long lines (N = 2048 .. 8192): variant 3 only, one line per CTA; their
 // instantiations live in csl_pass32_big.cu / csl_pass64_big.cu.
@@ -531,23 +514,64 @@ size_t pass_smem(int N, int wide, int lines) {
   return 0;
 }
 
-template <int NN>
-inline int pass_tpl_n(int wide) {
-  if constexpr (NN >= 512) {
-    if (wide == 1) return LineDst<float, NN, 1>::TPL;
-    if (wide == 2) return LineDst<float, NN, 2>::TPL;
+// entries of the extra twiddle tables of length N, and where a variant's begin
+template <typename T>
+inline int pass_tp_total(int N) {
+  if constexpr (sizeof(T) == 4) {
+    return line_tp_size(N, 0) + line_tp_size(N, 1);
+  } else {
+    switch (N) {
+#define CASE(NN) \
+  case NN: return fix_table_entries<NN, LineDst<double, NN, 0>::TPL>();
+      CASE(4) CASE(8) CASE(16) CASE(32) CASE(64) CASE(128) CASE(256)
+#undef CASE
+      case 512: return fix_table_entries<512, 64>() + fix_table_entries<512, 128>();
+      case 1024: return fix_table_entries<1024, 64>() + fix_table_entries<1024, 128>();
+      case 2048: return fix_table_entries<2048, BigShape<2048>::TPL>();
+      case 4096: return fix_table_entries<4096, BigShape<4096>::TPL>();
+      case 8192: return fix_table_entries<8192, BigShape<8192>::TPL>();
+    }
+    return 0;
   }
-  return LineDst<float, NN, 0>::TPL;
+}
+template <typename T>
+inline int pass_tp_offset(int N, int wide) {
+  if (sizeof(T) == 4) return wide == 1 || wide == 2 ? line_tp_size(N, 0) : 0;
+  // variants 0 and 1 have the same radices
+  return wide == 2 ? (N == 512 ? fix_table_entries<512, 64>() : fix_table_entries<1024, 64>()) : 0;
+}
+// the FP64 form's pass tables of length N, in the order of pass_tp_offset
+// (lines of 16384 points have none)
+inline FixRadices fix_radices_of(int N, int wide) {
+  switch (N) {
+    case 32: return fix_radices<32, LineDst<double, 32, 0>::TPL>();
+    case 64: return fix_radices<64, LineDst<double, 64, 0>::TPL>();
+    case 128: return fix_radices<128, LineDst<double, 128, 0>::TPL>();
+    case 256: return fix_radices<256, LineDst<double, 256, 0>::TPL>();
+    case 512: return wide == 2 ? fix_radices<512, 128>() : fix_radices<512, 64>();
+    case 1024: return wide == 2 ? fix_radices<1024, 128>() : fix_radices<1024, 64>();
+    case 2048: return fix_radices<2048, BigShape<2048>::TPL>();
+    case 4096: return fix_radices<4096, BigShape<4096>::TPL>();
+    case 8192: return fix_radices<8192, BigShape<8192>::TPL>();
+  }
+  return {0, {0, 0, 0, 0}};
 }
 
+// lanes per line of a variant
+template <typename T>
 inline int pass_tpl(int N, int wide) {
   switch (N) {
 #define BIGCASE(NN) \
-  case NN: return LineDst<float, NN, 3>::TPL;
+  case NN: return LineDst<T, NN, 3>::TPL;
     CSL_FOR_EACH_BIG_N(BIGCASE)
 #undef BIGCASE
-#define CASE(NN) \
-  case NN: return pass_tpl_n<NN>(wide);
+#define CASE(NN)                                       \
+  case NN:                                             \
+    if constexpr (NN >= 512) {                         \
+      if (wide == 1) return LineDst<T, NN, 1>::TPL;    \
+      if (wide == 2) return LineDst<T, NN, 2>::TPL;    \
+    }                                                  \
+    return LineDst<T, NN, 0>::TPL;
     CSL_FOR_EACH_N(CASE)
 #undef CASE
   }
@@ -562,6 +586,15 @@ cudaError_t launch_row(int N, int wide, int load, int store, const RowArgs<T>& a
 template <typename T>
 cudaError_t launch_strided(int N, int wide, bool mid, const StridedArgs<T>& a, const PassLaunch& L,
                            cudaStream_t s, const StridedArgs<T>* batch = nullptr, int nsys = 0);
+// one transform length and variant (csl_pass_impl.cuh)
+template <typename T, int N, int W>
+cudaError_t launch_row_n(int load, int store, const RowArgs<T>& a, const PassLaunch& L, cudaStream_t s,
+                         const RowArgs<T>* batch, int nsys);
+template <typename T, int N, int W>
+cudaError_t launch_strided_n(bool mid, const StridedArgs<T>& a, const PassLaunch& L, cudaStream_t s,
+                             const StridedArgs<T>* batch, int nsys);
+template <typename T, int N, int W>
+cudaError_t set_pass_attrs_n();
 // dynamic shared memory limit of one kernel = opt-in maximum - its static shared memory
 inline cudaError_t allow_dyn_smem(const void* k) {
   int dev = 0, optin = 0;

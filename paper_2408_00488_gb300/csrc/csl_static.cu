@@ -34,10 +34,13 @@ constexpr int kMaxN = 1024;                 // transform length n + 1
 constexpr int kMaxDevices = 64;
 
 // per-axis table sizes (in doubles): twiddles (N/2 complex), half sines
-// (N/2+1), extra twiddles (line_tp_size(N) complex), eigenvalues (n, FP64 and FP32)
+// (N/2+1), extra twiddles, eigenvalues (n, FP64 and FP32)
 constexpr int kTwD = kMaxN;                        // N/2 complex = N doubles
 constexpr int kHsD = kMaxN / 2 + 2;
-constexpr int kTpD = 2 * (8 * 8 + 8 * 8 * 16) + 2;  // largest line_tp_size (N = 1024), complex
+// extra twiddles, complex: the larger of the FP32 variant's and of the FP64 form's pass tables (N = 1024)
+constexpr int kTpE = wide_tp_size<1024>() > fix_table_entries<1024, 64>() ? wide_tp_size<1024>()
+                                                                           : fix_table_entries<1024, 64>();
+constexpr int kTpD = 2 * kTpE + 2;
 constexpr int kAxisD = kTwD + kHsD + kTpD + 2 * kMaxN;
 
 __device__ __align__(256) double g_static_T[2 * kStaticMaxPoints];     // intermediate (double2 / float2)
@@ -62,7 +65,7 @@ int ilog2_exact_s(long v) {
 
 // Tables of one axis, in the precision T, laid out in the axis slice:
 //   tw[m] = exp(-2 pi i m/N) (m < N/2), hs[j] = sin(pi j/N)/2 (j <= N/2),
-//   tp = extra twiddles (layout of LineDst<T,N>::TP), mu_d[k], mu_f[k]
+//   tp = extra twiddles (variant 1 at N >= 512), mu_d[k], mu_f[k]
 //   (mu_k = (4/h^2) sin^2(k pi / (2N)), k = 1..n, h = 1/N).
 template <typename T>
 struct AxisTables {
@@ -93,22 +96,28 @@ __device__ void root_of_unity(long num, long den, double& c, double& s) {
 }
 
 template <typename T>
-__global__ void k_static_axis_tables(double* tables, int N) {
+__global__ void k_static_axis_tables(double* tables, int N, FixRadices radices, int ntp) {
   AxisTables<T> a = axis_tables<T>(tables);
   const int H = N / 2, n = N - 1;
   const double h = 1.0 / (double)N;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N + 8 * 8 * 16 + 8 * 8 + 2; i += gridDim.x * blockDim.x) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N + kTpE; i += gridDim.x * blockDim.x) {
     double c, s;
-    if (i < H) {
-      root_of_unity(i, N, c, s);
-      a.tw[i] = mkc<T>((T)c, (T)s);
+    if constexpr (sizeof(T) == 8) {  // 64-bit fixed point (csl_fix.cuh): half sines and pass tables
+      if (i <= H) ((int2*)a.hs)[i] = fx_half_sine(i, N);
+      if (i < ntp) ((fxw*)a.tp)[i] = fix_table_entry(radices, i);
+    } else {
+      if (i < H) {
+        root_of_unity(i, N, c, s);
+        a.tw[i] = mkc<T>((T)c, (T)s);
+      }
+      if (i <= H) a.hs[i] = (T)(i == H ? 0.5 : 0.5 * sinpi((double)i / (double)N));
     }
-    if (i <= H) a.hs[i] = (T)(i == H ? 0.5 : 0.5 * sinpi((double)i / (double)N));
     if (i >= 1 && i <= n) {
       const double sn = sinpi((double)i / (2.0 * N));
       a.mu_d[i - 1] = 4.0 / (h * h) * sn * sn;
       a.mu_f[i - 1] = (float)a.mu_d[i - 1];
     }
+    if (sizeof(T) == 8) continue;
     // extra twiddles
     if (N >= 64 && N < 512) {
       int R1 = 0, R2 = 0;
@@ -167,7 +176,7 @@ void setup_device(int dev) {
 template <typename T>
 PassLaunch static_launch(int N, long nlines_or_tiles_per_cta_unit, bool strided, int ncols, int nouter) {
   const int wide = pass_has_wide(N) ? 1 : 0;
-  const int tpl = pass_tpl(N, wide);
+  const int tpl = pass_tpl<T>(N, wide);
   int threads = 256;
   if (strided)
     while (threads > 32 && threads > tpl && (threads / tpl) / 2 >= ncols) threads >>= 1;
@@ -245,7 +254,11 @@ cudaError_t run_static(int dim, const int n[3], double gamma, double alpha, doub
   for (int d = 0; d < dim; ++d) {
     const int N = n[d] + 1;
     cnorm *= 2.0 / (double)N;
-    k_static_axis_tables<T><<<8, 256, 0, s>>>(P.tables + (long)d * kAxisD, N);
+    const int wide = pass_has_wide(N) ? 1 : 0;
+    const FixRadices f = fix_radices_of(N, wide);
+    int ntp = 0;
+    for (int p = 1, ls = f.r[0]; p < f.np; ++p) ntp += (ls *= f.r[p]);
+    k_static_axis_tables<T><<<8, 256, 0, s>>>(P.tables + (long)d * kAxisD, N, f, ntp);
     ax[d] = axis_tables<T>(P.tables + (long)d * kAxisD);
   }
   cudaError_t e = cudaGetLastError();
