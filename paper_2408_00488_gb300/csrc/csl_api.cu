@@ -621,7 +621,7 @@ cudaError_t launch_precondition_T(csl_plan* P, const double2* v, double2* out, c
 
 // one kernel (index k of the iteration's sequence) of the MINRES iteration
 // with buffer parity par, on the plan's stream (measurement and tuning);
-// mid_mode: the MID pass's scalar tail (2: Givens step, 0: none)
+// mid_mode: the MID pass's scalar tail (2: Givens step, 3: the reduction alone)
 cudaError_t launch_iteration_kernel(csl_plan* P, int k, int par, int mid_mode) {
   const bool fp32 = P->precision != CSL_PREC_FP64;
   const int nkb = P->dim == 2 ? 4 : 6;  // kernels of the main chain
@@ -695,6 +695,9 @@ DevState scratch_state(const csl_plan* P) {
   DevState h;
   memset(&h, 0, sizeof(h));
   h.gam = h.gam_old = h.gam1 = 1.0;
+  h.inv_gam = h.lanc = 1.0;
+  h.lanc2 = make_float2(1.f, 0.f);
+  h.beta2 = make_float2((float)P->beta, (float)(P->beta - (double)(float)P->beta));
   h.a1inv_old = h.a1inv_old2 = 1.0;
   h.c = h.c_old = 1.0;
   h.eta = h.eta_x = h.bnorm = h.r0norm = 1.0;
@@ -709,7 +712,8 @@ DevState scratch_state(const csl_plan* P) {
 // Each sine-transform pass tries every CTA size and, for N = 512 and 1024,
 // every transform variant.  A candidate is timed inside the iteration's own
 // kernel sequence (time_sequence: three iterations after a warm-up, on
-// zeroed vectors and a scratch state, the MID pass without its scalar tail),
+// zeroed vectors and a scratch state, the MID pass with its reduction but
+// without the Givens step),
 // so that its cost includes the caches and the predecessor it really has;
 // the candidate with the smallest summed duration of the pass's kernels is
 // kept.  Results are cached per (precision, pass, geometry) for the life of
@@ -803,7 +807,7 @@ cudaError_t tune_pass(csl_plan* P, PassCfg& c, int kind, cudaEvent_t* ev, const 
       double t = 1e30;
       for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {  // the faster of two measurements
         e = cudaMemcpyAsync(P->st, &hst, sizeof(hst), cudaMemcpyHostToDevice, P->stream);
-        if (e == cudaSuccess) e = time_sequence(P, 3, 0, ev, ms);
+        if (e == cudaSuccess) e = time_sequence(P, 3, 3, ev, ms);
         double sum = 0.0;
         for (int i = 0; i < nidx; ++i) sum += ms[idx[i]];
         if (e == cudaSuccess && sum < t) t = sum;

@@ -177,9 +177,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kCThreads, 1) k_row_
   const int rank = (int)cl.block_rank();
   const int t = rank * kCThreads + (int)threadIdx.x;
   const int cid = (int)blockIdx.x / 2, ncl = (int)gridDim.x / 2;
-  const double lz = LOAD == LOAD_LANCZOS ? a.st->delta / a.st->gam : 0.0;
-  const double zs = ((STORE == STORE_Z || STORE == STORE_Z_UPDATE) && a.st) ? (a.st->gam > 0.0 ? 1.0 / a.st->gam : 0.0)
-                                                                               : 1.0;
+  const double lz = LOAD == LOAD_LANCZOS ? a.st->lz : 0.0;
+  const double zs = ((STORE == STORE_Z || STORE == STORE_Z_UPDATE) && a.st) ? a.st->inv_gam : 1.0;
   const double wb = STORE == STORE_Z_UPDATE ? a.st->w_b : 0.0, wc = STORE == STORE_Z_UPDATE ? a.st->w_c : 0.0;
   const double xc = STORE == STORE_Z_UPDATE ? a.st->x_coef : 0.0;
   const int n = a.n;

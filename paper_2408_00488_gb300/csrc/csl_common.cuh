@@ -79,7 +79,7 @@ template <> __device__ __forceinline__ float2 store_as<float2>(double2 v) {
 // Scalars of one MINRES solve, resident in device memory so that the whole
 // iteration (including the Givens step and the stopping decision) runs
 // without host round trips.
-struct DevState {
+struct alignas(16) DevState {
   // Lanczos recurrence: gam = gamma_j, gam_old = gamma_{j-1}, delta = delta_j
   double gam, gam_old, gam1, delta;
   // Givens rotations (c_j, c_{j-1}, s_j, s_{j-1}) and the rotated right-hand side eta
@@ -96,6 +96,13 @@ struct DevState {
   double beta;    // coupling coefficient of this solve (beta, or -beta for the adjoint)
   double sqrt_pmin, sqrt_pmax;  // sqrt of extreme eigenvalues of one block of P
   double r0norm;  // ||b - A x_0||_2 of the start vector (= bnorm for x_0 = 0)
+  // quotients every CTA of the following kernels needs, formed once by the
+  // scalar steps: an FP64 division in every warp holds the SM's FP64 pipe for
+  // about 160 clocks a warp
+  double lanc;     // gamma_j / gamma_{j-1}
+  double lz;       // delta_j / gamma_j
+  double inv_gam;  // 1 / gamma_j (0 for gamma_j = 0)
+  float2 lanc2, beta2;  // lanc and beta as float pairs
   double* hist;   // optional: |eta_j| / gamma_1 of every iteration j (hist_cap entries), or null
   int hist_cap;
   int entries;    // Givens steps started (MID passes): a loop bound that needs no reduction
@@ -104,18 +111,37 @@ struct DevState {
   unsigned int tickets[4];
 };
 
-static_assert(sizeof(DevState) % 4 == 0, "DevState is copied as 32-bit words");
+static_assert(sizeof(DevState) % 16 == 0, "DevState is copied as 16-byte words");
 
-// Copy of the solver state into shared memory, taken when a kernel starts
+// Asynchronous global -> shared copies (cp.async) of 8 or 16 bytes; a false
+// predicate copies nothing and zero-fills the destination (the source is
+// then not read, and callers pass a valid address anyway).
+__device__ __forceinline__ void cp_async8(void* dst, const void* src, bool pred) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(pred ? 8 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool pred) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(pred ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Copy of the solver state into shared memory, started when a kernel starts
 // (after its predecessor completed), so that the scalar step at its end does
 // not wait on a global round trip.  Only that step changes the scalars while
 // the kernel runs; the reduction tickets do change (other CTAs may have
 // arrived before this one started), so a scalar step writes back the fields
-// it sets, never the whole copy.  Block-wide; a barrier must separate it from
-// the reads.
+// it sets, never the whole copy.  Block-wide and asynchronous: it joins the
+// next cp.async group, and a wait for that group and a barrier must separate
+// it from the reads.  (Through registers, the warps' later loads would wait
+// for it.)
 __device__ __forceinline__ void state_prefetch(DevState* dst, const DevState* st) {
-  constexpr int W = (int)(sizeof(DevState) / 4);
-  for (int i = threadIdx.x; i < W; i += blockDim.x) ((unsigned*)dst)[i] = ((const unsigned*)st)[i];
+  constexpr int W = (int)(sizeof(DevState) / 16);
+  for (int i = threadIdx.x; i < W; i += blockDim.x) cp_async16((uint4*)dst + i, (const uint4*)st + i, true);
 }
 
 enum { TICKET_STENCIL = 0, TICKET_MID = 1, TICKET_INGEST = 2, TICKET_AUX = 3 };  // TICKET_AUX: warm start
@@ -135,76 +161,84 @@ enum {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Sum over the warp, valid in lane 0.  Only the lanes whose sum is still needed
+// add: the FP64 pipe takes two lanes a clock, so a full warp's addition holds
+// it for 16 clocks.
 __device__ __forceinline__ double warp_sum(double v) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  for (int o = 16; o > 0; o >>= 1) {
+    const double u = __shfl_down_sync(0xffffffffu, v, o);
+    if (lane < o) v += u;
+  }
   return v;
 }
 
-// Sum NV per-thread values over the block; result valid in thread 0.
+// Deterministic grid reduction of nv <= NV values per thread: every block
+// deposits its block sum in partials[bid*NV + i]; the last block to arrive
+// (atomic ticket) sums the deposits in block order.  Returns true in warp 0 of
+// that block only, with the totals in tot[] of all its lanes; every other warp
+// returns false.  The ticket is re-armed for reuse.
+// bid / nblk: the block's index and the number of blocks working on the same
+// system (the whole grid for a single system; one slice of a batched launch).
+//
+// FP64 sums hold the SM's FP64 pipe for 16 clocks per full-warp instruction
+// and take 67 clocks each in a chain.  So a warp folds its halves once, and
+// warp 0 alone adds the rest up from shared memory: 8 + 4 + 5 sums for a block
+// of 8 warps, where a shuffle tree in every warp took 45 and held the float-
+// pair stencil's last CTAs up by 2 us (n = 1023: 28.8 -> 24.6 us with the
+// state's quotients formed once).  At most 512 threads.
 template <int NV>
-__device__ __forceinline__ void block_sum(double (&v)[NV], double* sh /* >= 32*NV */) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+__device__ bool grid_sum_last_block(double (&v)[NV], double* partials, unsigned int* ticket,
+                                    double (&tot)[NV], int bid, int nblk, int nv = NV) {
+  __shared__ double sh[NV][256];
+  __shared__ int s_last;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, ns = (blockDim.x >> 5) * 16;
+  // value i's block sum, valid in lane 0 of warp 0
+  auto fold = [&](int i, double x) {
+    const double u = __shfl_down_sync(0xffffffffu, x, 16);
+    if (lane < 16) sh[i][wid * 16 + lane] = x + u;
+  };
+  auto finish = [&](int i) {
+    double t = lane < ns ? sh[i][lane] : 0.0;
+    for (int k = lane + 32; k < ns; k += 32) t += sh[i][k];
+    return warp_sum(t);
+  };
 #pragma unroll
-  for (int i = 0; i < NV; ++i) v[i] = warp_sum(v[i]);
-  __syncthreads();
-  if (lane == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) sh[wid * NV + i] = v[i];
-  }
+  for (int i = 0; i < NV; ++i)
+    if (i < nv) fold(i, v[i]);
   __syncthreads();
   if (wid == 0) {
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-      double t = (lane < nw) ? sh[lane * NV + i] : 0.0;
-      v[i] = warp_sum(t);
+      const double t = i < nv ? finish(i) : 0.0;
+      if (lane == 0) partials[bid * NV + i] = t;
+    }
+    if (lane == 0) {
+      // one acquire-release arrival: the release orders this thread's partial
+      // stores before it, and the last arrival's acquire orders every other
+      // CTA's partials before this CTA's reads below (the CTA barrier passes
+      // that order on to the other threads)
+      unsigned int t;
+      asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(t) : "l"(ticket) : "memory");
+      s_last = (t == (unsigned)nblk - 1);
     }
   }
   __syncthreads();
-}
-
-// Deterministic grid reduction: every block deposits its block sum in
-// partials[blockIdx.x*NV + i]; the last block to arrive (atomic ticket) sums
-// the deposits in block order and returns true with the totals in tot[]
-// (valid in all threads of that block).  The ticket is re-armed for reuse.
-// bid / nblk: the block's index and the number of blocks working on the same
-// system (the whole grid for a single system; one slice of a batched launch).
-template <int NV>
-__device__ bool grid_sum_last_block(double (&v)[NV], double* partials, unsigned int* ticket,
-                                    double (&tot)[NV], int bid, int nblk) {
-  __shared__ double sh[32 * NV];
-  __shared__ int s_last;
-  block_sum<NV>(v, sh);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) partials[bid * NV + i] = v[i];
-    // one acquire-release arrival: the release orders this thread's partial
-    // stores before it, and the last arrival's acquire orders every other
-    // CTA's partials before this CTA's reads below (the CTA barrier passes
-    // that order on to the other threads)
-    unsigned int t;
-    asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(t) : "l"(ticket) : "memory");
-    s_last = (t == (unsigned)nblk - 1);
-  }
-  __syncthreads();
   if (!s_last) return false;
-  double acc[NV];
 #pragma unroll
-  for (int i = 0; i < NV; ++i) acc[i] = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) acc[i] += ((volatile double*)partials)[b * NV + i];
-  }
-  block_sum<NV>(acc, sh);
-  __shared__ double s_tot[NV];
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) s_tot[i] = acc[i];
-    *ticket = 0u;
+  for (int i = 0; i < NV; ++i) {
+    if (i < nv) {
+      double acc = 0.0;
+      for (int b = threadIdx.x; b < nblk; b += blockDim.x) acc += __ldcg(partials + (size_t)b * NV + i);
+      fold(i, acc);
+    }
   }
   __syncthreads();
+  if (wid != 0) return false;
 #pragma unroll
-  for (int i = 0; i < NV; ++i) tot[i] = s_tot[i];
+  for (int i = 0; i < NV; ++i) tot[i] = i < nv ? __shfl_sync(0xffffffffu, finish(i), 0) : 0.0;
+  if (lane == 0) *ticket = 0u;
   return true;
 }
 

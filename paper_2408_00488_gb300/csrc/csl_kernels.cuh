@@ -370,23 +370,6 @@ struct StepOperands {
   }
 };
 
-// Asynchronous global -> shared copies (cp.async) of 8 or 16 bytes; a false
-// predicate copies nothing and zero-fills the destination (the source is
-// then not read, and callers pass a valid address anyway).
-__device__ __forceinline__ void cp_async8(void* dst, const void* src, bool pred) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(pred ? 8 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool pred) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(pred ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // Float-pair stencil: one stage of a warp's operand ring holds what step m of
 // its strip needs beyond the values carried from step m-1 (ẑ at m-1 and m,
 // in 2D the south face = the previous north face, in 3D the lower z-face =
@@ -431,29 +414,9 @@ __global__ void __launch_bounds__(256, FF ? (DIM == 2 ? 3 : 2) : 2)
   const int nblk = batch ? bps : (int)gridDim.x;
   const StencilArgs a = batch ? batch[sys] : a0;
   DevState* st = a.st;
+  __shared__ DevState s_pre;
   pdl_wait();
-  // `entries` counts the Givens steps (the MID pass of each iteration adds
-  // one; nothing changes it while this kernel runs, so every CTA reads the
-  // same value): a bound on the device-side loop that does not rely on the
-  // scalar step at the end of this pass
-  const bool over = st->entries > st->maxit + 8;
-  if (st->done || over) {
-    if (bid == 0 && threadIdx.x == 0) {
-      if (!st->done) {
-        st->status = ST_NOT_CONVERGED;
-        st->done = 1;
-      }
-      // keep the device-side loop closed whatever set `done`
-      if (a.use_cond) cudaGraphSetConditional(a.cond, 0u);
-    }
-    return;
-  }
-  __shared__ DevState s_pre;  // for the scalar step at the end
   state_prefetch(&s_pre, st);
-  // z_j arrives normalised (z_j / gamma_j), so A z_j needs no scaling
-  const double gam = st->gam, gam_old = st->gam_old, beta = st->beta;
-  const double lanc = gam / gam_old;
-  const int check = st->check;
   const TZ* z = (const TZ*)a.z;
   const int nx = a.g.nx, ny = a.g.ny;
   const int nm = DIM == 2 ? a.g.ny : a.g.nz;
@@ -466,66 +429,120 @@ __global__ void __launch_bounds__(256, FF ? (DIM == 2 ? 3 : 2) : 2)
   const unsigned nstrips = (unsigned)stencil_strips(DIM, nx, ny, a.g.nz, strip);
   double acc[2] = {0.0, 0.0};
   ff2 dacc = {0.f, 0.f};
-  float2 beta2 = make_float2(0.f, 0.f), lanc2 = make_float2(0.f, 0.f);
-  if (FF) {
-    beta2 = d_to_ff(beta);
-    lanc2 = d_to_ff(lanc);
-  }
-  for (unsigned s = (unsigned)bid * (blockDim.x >> 5) + (threadIdx.x >> 5); s < nstrips;
-       s += (unsigned)nblk * (blockDim.x >> 5)) {
+  // one strip: its first column and its steps m0 .. m1
+  struct Strip {
+    int x, m0, m1, yfix;
+    bool vx;
+    long base;
+  };
+  auto strip_at = [&](unsigned s) {
+    Strip t;
     const unsigned q = s / nsx;  // 2D: q < nsm; 3D: q = yfix * nsm + sm
-    const int sx = (int)(s - q * nsx);
     const int sm = DIM == 3 ? (int)(q % nsm) : (int)q;
-    const int yfix = DIM == 3 ? (int)(q / nsm) : 0;
-    const int x = sx * 32 + lane;
-    const bool vx = x < nx;
-    const int m0 = sm * strip, m1 = min(m0 + strip, nm);
-    const long base = DIM == 2 ? (long)x : (long)yfix * nx + x;
-    if (FF && !check) {
-      // Operands stream through the warp's ring of kFFStages stages, filled
-      // kFFStages - 1 steps ahead by cp.async; ẑ at m-1 and m and the faces
-      // shared with the previous step are carried in registers.
-      const float2* zf = (const float2*)a.z;
-      const float2 zero = make_float2(0.f, 0.f);
-      const float2 nbeta2 = make_float2(-beta2.x, -beta2.y);
-      extern __shared__ __align__(16) unsigned char ff_ring[];
-      unsigned char* ring = ff_ring + (size_t)(threadIdx.x >> 5) * kFFStages * ff_stage_bytes<DIM>();
-      const int nsteps = m1 - m0;
-      auto issue = [&](int m, int slot) {
-        FFStage<DIM>& S = *(FFStage<DIM>*)(ring + slot * ff_stage_bytes<DIM>());
-        const long p = base + (long)m * mstride;
-        long rx, ry;
-        if (DIM == 2) {
-          rx = (long)m * (nx + 1) + x;
-          ry = (long)m * nx + x;
-        } else {
-          rx = ((long)m * ny + yfix) * (nx + 1) + x;
-          ry = ((long)m * (ny + 1) + yfix) * nx + x;
-        }
-        cp_async16(&S.v[lane], vx ? (const void*)(a.vold + p) : (const void*)a.vold, vx);
-        const bool hz = vx && m + 1 < nm;
-        cp_async8(&S.zp[lane], hz ? zf + p + mstride : zf, hz);
-        cp_async8(&S.cn[lane], vx ? a.cyp + ry + nx : a.cyp, vx);
-        const bool hw = x <= nx;  // the face left of column x exists for x = nx too
-        cp_async8(&S.cw[lane], hw ? a.cxp + rx : a.cxp, hw);
-        if (lane == 31) cp_async8(&S.cw[32], vx ? a.cxp + rx + 1 : a.cxp, vx);
-        if (lane == 0) cp_async8(&S.edge[0], (vx && x > 0) ? zf + p - 1 : zf, vx && x > 0);
-        if (lane == 31) cp_async8(&S.edge[1], (x + 1 < nx) ? zf + p + 1 : zf, x + 1 < nx);
-        if (DIM == 3) {
-          cp_async8(&S.cs[lane], vx ? a.cyp + ry : a.cyp, vx);
-          const bool hs = vx && yfix > 0, hn = vx && yfix < ny - 1;
-          cp_async8(&S.ys[lane], hs ? zf + p - nx : zf, hs);
-          cp_async8(&S.yn[lane], hn ? zf + p + nx : zf, hn);
-          cp_async8(&S.cu[lane], vx ? a.czp + p + mstride : a.czp, vx);
-        }
-      };
-      // prologue: stages for steps m0 .. m0 + kFFStages - 2 (one group each,
-      // empty groups past the strip's end keep the group count uniform)
+    t.yfix = DIM == 3 ? (int)(q / nsm) : 0;
+    t.x = (int)(s - q * nsx) * 32 + lane;
+    t.vx = t.x < nx;
+    t.m0 = sm * strip;
+    t.m1 = min(t.m0 + strip, nm);
+    t.base = DIM == 2 ? (long)t.x : (long)t.yfix * nx + t.x;
+    return t;
+  };
+  // float-pair path: operands stream through the warp's ring of kFFStages
+  // stages, filled kFFStages - 1 steps ahead by cp.async
+  const float2* zf = (const float2*)a.z;
+  const float2 fzero = make_float2(0.f, 0.f);
+  extern __shared__ __align__(16) unsigned char ff_ring[];
+  unsigned char* ring = ff_ring + (size_t)(threadIdx.x >> 5) * kFFStages * ff_stage_bytes<DIM>();
+  auto issue = [&](const Strip& t, int m, int slot) {
+    const int x = t.x, yfix = t.yfix;
+    const bool vx = t.vx;
+    FFStage<DIM>& S = *(FFStage<DIM>*)(ring + slot * ff_stage_bytes<DIM>());
+    const long p = t.base + (long)m * mstride;
+    long rx, ry;
+    if (DIM == 2) {
+      rx = (long)m * (nx + 1) + x;
+      ry = (long)m * nx + x;
+    } else {
+      rx = ((long)m * ny + yfix) * (nx + 1) + x;
+      ry = ((long)m * (ny + 1) + yfix) * nx + x;
+    }
+    cp_async16(&S.v[lane], vx ? (const void*)(a.vold + p) : (const void*)a.vold, vx);
+    const bool hz = vx && m + 1 < nm;
+    cp_async8(&S.zp[lane], hz ? zf + p + mstride : zf, hz);
+    cp_async8(&S.cn[lane], vx ? a.cyp + ry + nx : a.cyp, vx);
+    const bool hw = x <= nx;  // the face left of column x exists for x = nx too
+    cp_async8(&S.cw[lane], hw ? a.cxp + rx : a.cxp, hw);
+    if (lane == 31) cp_async8(&S.cw[32], vx ? a.cxp + rx + 1 : a.cxp, vx);
+    if (lane == 0) cp_async8(&S.edge[0], (vx && x > 0) ? zf + p - 1 : zf, vx && x > 0);
+    if (lane == 31) cp_async8(&S.edge[1], (x + 1 < nx) ? zf + p + 1 : zf, x + 1 < nx);
+    if (DIM == 3) {
+      cp_async8(&S.cs[lane], vx ? a.cyp + ry : a.cyp, vx);
+      const bool hs = vx && yfix > 0, hn = vx && yfix < ny - 1;
+      cp_async8(&S.ys[lane], hs ? zf + p - nx : zf, hs);
+      cp_async8(&S.yn[lane], hn ? zf + p + nx : zf, hn);
+      cp_async8(&S.cu[lane], vx ? a.czp + p + mstride : a.czp, vx);
+    }
+  };
+  // the stages of a strip's first kFFStages - 1 steps (one group each, empty
+  // groups past the strip's end keep the group count uniform)
+  auto fill = [&](const Strip& t) {
 #pragma unroll
-      for (int k = 0; k < kFFStages - 1; ++k) {
-        if (k < nsteps) issue(m0 + k, k);
-        cp_async_commit();
+    for (int k = 0; k < kFFStages - 1; ++k) {
+      if (k < t.m1 - t.m0) issue(t, t.m0 + k, k);
+      cp_async_commit();
+    }
+  };
+  unsigned s = (unsigned)bid * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const unsigned sstep = (unsigned)nblk * (blockDim.x >> 5);
+  bool filled = false;
+  if constexpr (FF) {  // the first strip's operands travel while the state does
+    if (s < nstrips) {
+      fill(strip_at(s));
+      filled = true;
+    }
+  }
+  if (filled) {
+    cp_async_wait<kFFStages - 2>();  // the state came with the first stage
+  } else {
+    cp_async_commit();
+    cp_async_wait<0>();
+  }
+  __syncthreads();  // s_pre
+  // `entries` counts the Givens steps (the MID pass of each iteration adds
+  // one; nothing changes it while this kernel runs, so every CTA reads the
+  // same value): a bound on the device-side loop that does not rely on the
+  // scalar step at the end of this pass
+  const bool over = s_pre.entries > s_pre.maxit + 8;
+  if (s_pre.done || over) {
+    if (FF) cp_async_wait<0>();
+    if (bid == 0 && threadIdx.x == 0) {
+      if (!s_pre.done) {
+        st->status = ST_NOT_CONVERGED;
+        st->done = 1;
       }
+      // keep the device-side loop closed whatever set `done`
+      if (a.use_cond) cudaGraphSetConditional(a.cond, 0u);
+    }
+    return;
+  }
+  // z_j arrives normalised (z_j / gamma_j), so A z_j needs no scaling
+  const double beta = s_pre.beta, lanc = s_pre.lanc;
+  const int check = s_pre.check;
+  const float2 beta2 = s_pre.beta2, lanc2 = s_pre.lanc2;
+  if (FF && check) cp_async_wait<0>();  // the checking pass does not use the ring
+  for (; s < nstrips; s += sstep) {
+    const Strip t = strip_at(s);
+    const int x = t.x, m0 = t.m0, m1 = t.m1, yfix = t.yfix;
+    const bool vx = t.vx;
+    const long base = t.base;
+    if (FF && !check) {
+      // ẑ at m-1 and m and the faces shared with the previous step are carried
+      // in registers
+      const float2 zero = fzero;
+      const float2 nbeta2 = make_float2(-beta2.x, -beta2.y);
+      const int nsteps = m1 - m0;
+      if (!filled) fill(t);
+      filled = false;
       const long p0 = base + (long)m0 * mstride;
       float2 zm = (vx && m0 > 0) ? zf[p0 - mstride] : zero;
       float2 zc = vx ? zf[p0] : zero;
@@ -540,7 +557,7 @@ __global__ void __launch_bounds__(256, FF ? (DIM == 2 ? 3 : 2) : 2)
       for (int i = 0; i < nsteps; ++i) {
         const int m = m0 + i;
         const long p = base + (long)m * mstride;
-        if (i + kFFStages - 1 < nsteps) issue(m + kFFStages - 1, (i + kFFStages - 1) % kFFStages);
+        if (i + kFFStages - 1 < nsteps) issue(t, m + kFFStages - 1, (i + kFFStages - 1) % kFFStages);
         cp_async_commit();
         cp_async_wait<kFFStages - 1>();
         __syncwarp();
@@ -670,7 +687,7 @@ __global__ void __launch_bounds__(256, FF ? (DIM == 2 ? 3 : 2) : 2)
   if (FF) acc[0] += ff_to_d(dacc);
   pdl_trigger();
   double tot[2];
-  if (!grid_sum_last_block<2>(acc, a.partials, &st->tickets[TICKET_STENCIL], tot, bid, nblk)) return;
+  if (!grid_sum_last_block<2>(acc, a.partials, &st->tickets[TICKET_STENCIL], tot, bid, nblk, check ? 2 : 1)) return;
   if (threadIdx.x != 0) return;
   // scalar step after the stencil: delta_j and the stopping test for x_{iter}.
   // It runs on a register copy of the state, loaded once and stored once: a
@@ -678,6 +695,10 @@ __global__ void __launch_bounds__(256, FF ? (DIM == 2 ? 3 : 2) : 2)
   // trip per dependent access on this single thread.
   DevState q = s_pre;
   q.delta = tot[0];
+  {  // delta / gamma from the stored reciprocal, one correction step
+    const double t = q.delta * q.inv_gam;
+    q.lz = fma(fma(-t, q.gam, q.delta), q.inv_gam, t);
+  }
   if (check) {
     const double rnorm = sqrt(tot[1]);
     const double rel = rnorm / q.bnorm;
@@ -703,6 +724,7 @@ __global__ void __launch_bounds__(256, FF ? (DIM == 2 ? 3 : 2) : 2)
   if (q.iter > q.maxit + 1 || q.loops > q.maxit + 4) q.done = 1;  // hard caps (integers only)
   // the fields this step sets (the copy's tickets and entry count may be stale)
   st->delta = q.delta;
+  st->lz = q.lz;
   st->relres = q.relres;
   st->checks = q.checks;
   st->check = q.check;
@@ -755,6 +777,9 @@ __device__ __forceinline__ void store_scalar_fields(DevState* st, const DevState
   st->gam_old = q.gam_old;
   st->gam = q.gam;
   st->gam1 = q.gam1;
+  st->inv_gam = q.inv_gam;
+  st->lanc = q.lanc;
+  st->lanc2 = q.lanc2;
   st->rho = q.rho;
   st->iter = q.iter;
   st->check = q.check;
@@ -763,23 +788,27 @@ __device__ __forceinline__ void store_scalar_fields(DevState* st, const DevState
   st->done = q.done;
 }
 
-// st: the caller's register copy of the solver state (see mid_scalar_tail).
-// It runs on one thread, where FP64 is latency-bound on GB300 (a dependent
-// FMA about 67 cycles, a division about 440, a square root about 700), so
-// the chain is kept short: a1 = sqrt(a0^2 + g2) does not wait for gn =
-// sqrt(g2), one reciprocal 1/a1 serves cn, sn and the x coefficient, and the
-// reciprocals of the last two a1 are kept in the state for the w coefficients.
+// st: the caller's register copy of the solver state (see mid_scalar_tail),
+// the same in every calling lane.  FP64 is latency-bound here (a
+// dependent FMA about 67 cycles, a division about 440, a square root about
+// 700), so the chain is kept short: a1 = sqrt(a0^2 + g2) does not wait for
+// gn = sqrt(g2), one reciprocal 1/a1 serves cn, sn and the x coefficient, the
+// reciprocals of the last two a1 are kept in the state for the w
+// coefficients, and lanes 0 to 2, which call this, take one square root and
+// one division each (two and three different ones) in the time of one.  More
+// lanes would hold the FP64 pipe longer: it takes two a clock.
 __device__ inline void givens_step(DevState* st, double g2) {
   if (!(g2 >= 0.0) || !(g2 < 1e300)) {
     st->done = 1;
     st->status = ST_BREAKDOWN;
     return;
   }
+  const int lane = threadIdx.x & 31;
   const double gam = st->gam, delta = st->delta;
   const double c = st->c, c_old = st->c_old, s = st->s, s_old = st->s_old;
   const double a0 = c * delta - c_old * s * gam;
-  const double gn = sqrt(g2);
-  const double a1 = sqrt(fma(a0, a0, g2));
+  const double root = sqrt(lane == 0 ? g2 : fma(a0, a0, g2));
+  const double gn = __shfl_sync(0x7u, root, 0), a1 = __shfl_sync(0x7u, root, 1);
   const double a2 = s * delta + c_old * c * gam;
   const double a3 = s_old * gam;
   // w_{j+1} = (z_j - a3 w_{j-1} - a2 w_j) / a1 with z_j stored normalised
@@ -792,7 +821,12 @@ __device__ inline void givens_step(DevState* st, double g2) {
     st->status = ST_BREAKDOWN;
     return;
   }
-  const double inv = 1.0 / a1;
+  // lane 0: 1 / gn, lane 1: gn / gam, lane 2: 1 / a1
+  const double quot = (lane == 1 ? gn : 1.0) / (lane == 0 ? gn : lane == 1 ? gam : a1);
+  const double inv = __shfl_sync(0x7u, quot, 2);
+  st->inv_gam = gn > 0.0 ? __shfl_sync(0x7u, quot, 0) : 0.0;
+  st->lanc = __shfl_sync(0x7u, quot, 1);
+  st->lanc2 = d_to_ff(st->lanc);
   const double cn = a0 * inv, sn = gn * inv;
   st->w_a = 1.0;
   st->w_b = wb;
@@ -811,7 +845,7 @@ __device__ inline void givens_step(DevState* st, double g2) {
   // stopping-test schedule for x_iter (evaluated by the next stencil pass)
   const double e = fabs(st->eta);
   st->eta_x = e;
-  if (st->hist && st->iter <= st->hist_cap) st->hist[st->iter - 1] = e / st->gam1;
+  if (st->hist && st->iter <= st->hist_cap && lane == 0) st->hist[st->iter - 1] = e / st->gam1;
   const double target = st->tol * st->bnorm;
   const double pred = st->rho * e;  // predicted ||b - A x||_2
   int chk = 0;
@@ -988,6 +1022,10 @@ static __global__ void __launch_bounds__(256) k_ingest(IngestArgs a0, const Inge
   st->s = st->s_old = 0.0;
   st->delta = 0.0;
   st->gam = st->gam_old = st->gam1 = 1.0;
+  st->lz = 0.0;
+  st->inv_gam = st->lanc = 1.0;
+  st->lanc2 = make_float2(1.f, 0.f);
+  st->beta2 = d_to_ff(a.beta);
   st->a1inv_old = st->a1inv_old2 = 1.0;
   st->eta = st->eta_x = 0.0;
   st->rho = 0.0;

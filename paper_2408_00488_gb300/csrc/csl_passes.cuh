@@ -76,7 +76,7 @@ struct StridedArgs {
   T gamma, alpha, beta2, cnorm;
   DevState* st;
   double* partials;
-  int scalar_mode;     // 0 none, 1 init (gamma_1), 2 MINRES iteration
+  int scalar_mode;     // 0 none, 1 init (gamma_1), 2 MINRES iteration, 3 the reduction alone (tuning)
   const void* sine_tc; // tensor-core variant: split-bf16 sine matrix in B-operand layout
 };
 
@@ -124,13 +124,15 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_ROW_MINB(T, N
   c_t* lines = s_scr + D::SCRATCH * nlines;
   const auto tb = D::Tables::load(smem_raw, a.tw, a.hs, a.tp);  // constant: may overlap the predecessor
   pdl_wait();
-  if (a.st && a.st->done) return;
+  // the state is read together with the first rows' data (one round trip);
+  // a finished solve leaves before anything is stored
+  const int done = a.st ? a.st->done : 0;
   double lz = 0.0, wb = 0.0, wc = 0.0, xc = 0.0;
-  if (LOAD == LOAD_LANCZOS) lz = a.st->delta / a.st->gam;
+  if (LOAD == LOAD_LANCZOS) lz = a.st->lz;
   // MINRES works with the normalised z_{j+1} / gamma_{j+1}; gamma_{j+1} is
   // known once the MID pass has run, so the z store applies it
   T zs = (T)1;
-  if ((STORE == STORE_Z || STORE == STORE_Z_UPDATE) && a.st) zs = (T)(a.st->gam > 0.0 ? 1.0 / a.st->gam : 0.0);
+  if ((STORE == STORE_Z || STORE == STORE_Z_UPDATE) && a.st) zs = (T)a.st->inv_gam;
   float2 wb2 = make_float2(0.f, 0.f), wc2 = wb2, xc2 = wb2;
   if (STORE == STORE_Z_UPDATE) {
     wb = a.st->w_b;
@@ -166,6 +168,7 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_ROW_MINB(T, N
       }
       cp_async_commit();
       cp_async_wait<0>();
+      if (done) return;
     }
     // global loads in batches of UB elements per lane, all issued before use
 #pragma unroll
@@ -184,6 +187,7 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_ROW_MINB(T, N
             vc[k] = ((const float4*)a.vcur)[base + j];
           }
         }
+        if (done) return;
 #pragma unroll
         for (int k = 0; k < UB; ++k) {
           const int j = t + TPL * (i0 + k);
@@ -213,6 +217,7 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_ROW_MINB(T, N
             vc[k] = a.vcur[base + j];
           }
         }
+        if (done) return;
 #pragma unroll
         for (int k = 0; k < UB; ++k) {
           const int j = t + TPL * (i0 + k);
@@ -234,6 +239,7 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_ROW_MINB(T, N
           val[k] = mkc<T>((T)0, (T)0);
           if (valid && j < n) val[k] = (LOAD == LOAD_V) ? from_d2<T>(a.vin[base + j]) : a.tin[base + j];
         }
+        if (done) return;
 #pragma unroll
         for (int k = 0; k < UB; ++k) {
           const int j = t + TPL * (i0 + k);
@@ -316,8 +322,9 @@ template <typename T>
 __device__ void mid_scalar_tail(const StridedArgs<T>& a, double g2acc, int bid, int nblk,
                                 const DevState* pre = nullptr) {
   double v[1] = {g2acc}, tot[1];
+  // three lanes of the last CTA go on, each with the same state (givens_step)
   if (!grid_sum_last_block<1>(v, a.partials, &a.st->tickets[TICKET_MID], tot, bid, nblk)) return;
-  if (threadIdx.x != 0) return;
+  if (threadIdx.x > 2 || a.scalar_mode == 3) return;  // 3: tuning: the cost of the reduction, not its result
   // the scalar step runs on a register copy of the state and stores the
   // fields it sets
   DevState q = pre ? *pre : *a.st;
@@ -332,6 +339,9 @@ __device__ void mid_scalar_tail(const StridedArgs<T>& a, double g2acc, int bid, 
       q.gam = sqrt(g2);
       q.gam1 = q.gam;
       q.gam_old = 1.0;
+      q.lanc = q.gam;
+      q.lanc2 = d_to_ff(q.gam);
+      q.inv_gam = 1.0 / q.gam;
       q.eta = q.gam;
       q.eta_x = q.gam;
       q.rho = q.r0norm / q.gam;  // exact at the start vector
@@ -339,6 +349,7 @@ __device__ void mid_scalar_tail(const StridedArgs<T>& a, double g2acc, int bid, 
   } else {
     givens_step(&q, tot[0]);
   }
+  if (threadIdx.x != 0) return;
   store_scalar_fields(a.st, q);
 }
 
@@ -376,10 +387,11 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_PASS_MINB(T, 
   c_t* lines = s_scr + D::SCRATCH * C;
   const auto tb = D::Tables::load(smem_raw, a.tw, a.hs, a.tp);  // constant: may overlap the predecessor
   pdl_wait();
-  if (a.st && a.st->done) return;
   __shared__ DevState s_pre;
   if (MID && a.scalar_mode != 0) state_prefetch(&s_pre, a.st);
-  if (MID && a.scalar_mode == 2 && bid == 0 && threadIdx.x == 0) a.st->entries += 1;  // read by the next stencil pass
+  // read together with the first tile (one round trip); a finished solve
+  // leaves before anything is stored
+  const int done = a.st ? a.st->done : 0;
   int logC = 0;
   while ((1 << logC) < C) ++logC;
   const int myl = threadIdx.x / TPL, t = threadIdx.x - myl * TPL;
@@ -388,6 +400,7 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_PASS_MINB(T, 
   const int ntx = (a.ncols + C - 1) / C;
   const int ntiles = ntx * a.nouter;
   double g2acc = 0.0;
+  if (MID && a.scalar_mode == 2 && bid == 0 && threadIdx.x == 0 && !done) a.st->entries += 1;  // read by the next stencil pass
   for (int tile = bid; tile < ntiles; tile += nblk) {
     const int o = tile / ntx;
     const int col0 = (tile - o * ntx) * C;
@@ -412,6 +425,7 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_PASS_MINB(T, 
     }
     cp_async_commit();
     cp_async_wait<0>();
+    if (done) return;
     __syncthreads();
     if constexpr (MID && sizeof(T) == 8) {
       // the scale and the Parseval sum are applied to the results while they
@@ -466,6 +480,7 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_PASS_MINB(T, 
     }
   }
   pdl_trigger();
+  if (done) return;
   if (MID && a.scalar_mode != 0) mid_scalar_tail<T>(a, g2acc, bid, nblk, &s_pre);
 }
 

@@ -192,10 +192,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const int bid = batch ? (int)blockIdx.x - sys * bps : (int)blockIdx.x;
   const int nblk = batch ? bps : (int)gridDim.x;
   const StridedArgs<float> a = batch ? batch[sys] : a0;
-  pdl_wait();
-  if (a.st && a.st->done) return;
-  if (MID && a.scalar_mode == 2 && bid == 0 && threadIdx.x == 0) a.st->entries += 1;  // read by the next stencil pass
-
   extern __shared__ __align__(128) unsigned char tc_smem[];
   unsigned char* sB = tc_smem;                  // SPLIT sine-matrix terms
   unsigned char* sA = tc_smem + SPLIT * B_BYTES;  // SPLIT data terms
@@ -203,11 +199,17 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   __shared__ __align__(8) unsigned long long s_bar;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  {
+  {  // constant: may overlap the predecessor
     const uint4* src = (const uint4*)a.sine_tc;
     uint4* dst = (uint4*)sB;
     for (int i = tid; i < (int)(SPLIT * B_BYTES / 16); i += kTcThreads) dst[i] = src[i];
   }
+  pdl_wait();
+  if (a.st && a.st->done) return;
+  if (MID && a.scalar_mode == 2 && bid == 0 && threadIdx.x == 0) a.st->entries += 1;  // read by the next stencil pass
+  __shared__ DevState s_pre;
+  if (MID && a.scalar_mode != 0) state_prefetch(&s_pre, a.st);  // read by the scalar step
+  cp_async_commit();
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
                  "r"(TCOLS));
@@ -380,6 +382,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     tc_fence_after();
   }
   pdl_trigger();
+  cp_async_wait<0>();
   tc_fence_before();
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS));
@@ -387,7 +390,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     a.st->status = ST_TIMEOUT;
     a.st->done = 1;
   }
-  if (MID && a.scalar_mode != 0) mid_scalar_tail<float>(a, g2acc, bid, nblk);
+  if (MID && a.scalar_mode != 0) mid_scalar_tail<float>(a, g2acc, bid, nblk, &s_pre);
 }
 
 // ---------------------------------------------------------------------------
