@@ -102,7 +102,7 @@ struct alignas(16) DevState {
   double lanc;     // gamma_j / gamma_{j-1}
   double lz;       // delta_j / gamma_j
   double inv_gam;  // 1 / gamma_j (0 for gamma_j = 0)
-  float2 lanc2, beta2;  // lanc and beta as float pairs
+  float2 lanc2, beta2, lz2, wb2, wc2, xc2;  // lanc, beta, lz, w_b, w_c and x_coef as float pairs
   double* hist;   // optional: |eta_j| / gamma_1 of every iteration j (hist_cap entries), or null
   int hist_cap;
   int entries;    // Givens steps started (MID passes): a loop bound that needs no reduction

@@ -139,9 +139,9 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_ROW_MINB(T, N
     wc = a.st->w_c;
     xc = a.st->x_coef;
     if (pairs) {
-      wb2 = d_to_ff(wb);
-      wc2 = d_to_ff(wc);
-      xc2 = d_to_ff(xc);
+      wb2 = a.st->wb2;
+      wc2 = a.st->wc2;
+      xc2 = a.st->xc2;
     }
   }
   __syncthreads();
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_ROW_MINB(T, N
         // v_{j+1} = u' - (delta/gamma) v_j in pair arithmetic, stored
         // renormalised, its hi parts (= RN of the pair) feed the transform
         float4 u[UB], vc[UB];
-        const float2 lz2 = d_to_ff(lz);
+        const float2 lz2 = a.st->lz2;
 #pragma unroll
         for (int k = 0; k < UB; ++k) {
           const int j = t + TPL * (i0 + k);
@@ -322,9 +322,9 @@ template <typename T>
 __device__ void mid_scalar_tail(const StridedArgs<T>& a, double g2acc, int bid, int nblk,
                                 const DevState* pre = nullptr) {
   double v[1] = {g2acc}, tot[1];
-  // three lanes of the last CTA go on, each with the same state (givens_step)
+  // four lanes of the last CTA go on, each with the same state (givens_step)
   if (!grid_sum_last_block<1>(v, a.partials, &a.st->tickets[TICKET_MID], tot, bid, nblk)) return;
-  if (threadIdx.x > 2 || a.scalar_mode == 3) return;  // 3: tuning: the cost of the reduction, not its result
+  if (threadIdx.x > 3 || a.scalar_mode == 3) return;  // 3: tuning: the cost of the reduction, not its result
   // the scalar step runs on a register copy of the state and stores the
   // fields it sets
   DevState q = pre ? *pre : *a.st;
@@ -340,7 +340,6 @@ __device__ void mid_scalar_tail(const StridedArgs<T>& a, double g2acc, int bid, 
       q.gam1 = q.gam;
       q.gam_old = 1.0;
       q.lanc = q.gam;
-      q.lanc2 = d_to_ff(q.gam);
       q.inv_gam = 1.0 / q.gam;
       q.eta = q.gam;
       q.eta_x = q.gam;
@@ -348,6 +347,11 @@ __device__ void mid_scalar_tail(const StridedArgs<T>& a, double g2acc, int bid, 
     }
   } else {
     givens_step(&q, tot[0]);
+  }
+  if constexpr (sizeof(T) == 4) {  // the float pairs of the pair-vector forms, one a lane
+    const int l = threadIdx.x;
+    const float2 v = d_to_ff(l == 0 ? q.lanc : l == 1 ? q.w_b : l == 2 ? q.w_c : q.x_coef);
+    (l == 0 ? a.st->lanc2 : l == 1 ? a.st->wb2 : l == 2 ? a.st->wc2 : a.st->xc2) = v;
   }
   if (threadIdx.x != 0) return;
   store_scalar_fields(a.st, q);
