@@ -103,7 +103,7 @@ typedef struct csl_plan_options {
   int update_mode;         /* where the MINRES w/x update of an iteration runs: 0 (default) or
                              1: its own kernel on a side branch beside the inverse x transform;
                              2: fused into the inverse x transform; 3: its own kernel after
-                             the inverse x transform (batches always fuse)                  */
+                             the inverse x transform (batches: always as 3)                 */
   int body_iters;          /* MINRES iterations per body of the CUDA graph's WHILE loop: 0
                              (default) = 2, else 2, 4 or 8 (more amortise the loop's
                              per-body cost; up to body_iters - 1 iterations after

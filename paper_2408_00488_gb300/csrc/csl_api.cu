@@ -442,6 +442,12 @@ StencilArgs stencil_args(const csl_plan* P, int par) {
   return a;
 }
 
+// CTAs of the stencil: one warp per strip, 8 warps per CTA
+int stencil_blocks(const csl_plan* P, int strip) {
+  const long blocks = (stencil_strips(P->dim, P->n[0], P->n[1], P->n[2], strip) + 7) / 8;
+  return (int)(blocks < kSMs * 8 ? blocks : kSMs * 8);
+}
+
 typedef void (*StencilFn)(StencilArgs, const StencilArgs*, int);
 
 // the stencil kernel for the plan's form: float-pair arithmetic (ff) and
@@ -491,8 +497,7 @@ RowArgs<T> p3_args(csl_plan* P, int par) {
 }
 
 // the w/x update of the iteration with parity par (see k_update)
-template <typename T>
-cudaError_t launch_update(csl_plan* P, int par, cudaStream_t s) {
+UpdateArgs update_args(const csl_plan* P, int par) {
   UpdateArgs u;
   u.z = P->z[par];
   u.wprev = P->w[par];
@@ -500,13 +505,19 @@ cudaError_t launch_update(csl_plan* P, int par, cudaStream_t s) {
   u.x = P->x;
   u.st = P->st;
   u.M = P->M;
+  return u;
+}
+
+template <typename T>
+cudaError_t launch_update(csl_plan* P, int par, cudaStream_t s, const UpdateArgs* batch = nullptr, int nsys = 1) {
+  const UpdateArgs u = update_args(P, par);
   if constexpr (sizeof(T) == 4) {
     if (P->vpair) {
-      k_update<float2, true><<<P->upd_blocks, 256, 0, s>>>(u);
+      k_update<float2, true><<<P->upd_blocks * nsys, 256, 0, s>>>(u, batch, P->upd_blocks);
       return cudaGetLastError();
     }
   }
-  k_update<typename C2<T>::t, false><<<P->upd_blocks, 256, 0, s>>>(u);
+  k_update<typename C2<T>::t, false><<<P->upd_blocks * nsys, 256, 0, s>>>(u, batch, P->upd_blocks);
   return cudaGetLastError();
 }
 
@@ -1198,11 +1209,9 @@ csl_status csl_plan_create(csl_plan** out, int dim, const int64_t n[3], const do
     }
   }
   {
-    // one warp per strip, 8 warps per CTA
-    P->sten_strip = P->ff ? strip_rows(dim, nx, ny, nz, kSMs, 24)
-                    : dim == 2 ? strip_rows(dim, nx, ny, nz, kSMs, 16) : kStencilStrip;
-    const long blocks = (stencil_strips(dim, nx, ny, nz, P->sten_strip) + 7) / 8;
-    P->sten_blocks = (int)(blocks < kSMs * 8 ? blocks : kSMs * 8);
+    P->sten_strip = P->ff ? strip_rows(dim, nx, ny, nz, kSMs * 24)
+                    : dim == 2 ? strip_rows(dim, nx, ny, nz, kSMs * 16) : kStencilStrip;
+    P->sten_blocks = stencil_blocks(P, P->sten_strip);
   }
   Grid g;
   g.nx = nx;
@@ -1637,6 +1646,8 @@ struct BatchGroup {
   std::vector<int> sys;  // indices of the group's systems
   csl_plan* proto = nullptr;
   int ff = 1;  // all systems of the group take the float-pair stencil
+  int sten_strip = 1, sten_blocks = 1;  // the stencil's strips per system
+  UpdateArgs* d_upd[2] = {nullptr, nullptr};
   StencilArgs* d_sten[2] = {nullptr, nullptr};
   void* d_p1[2] = {nullptr, nullptr};   // RowArgs<T>
   void* d_p3[2] = {nullptr, nullptr};   // RowArgs<T>
@@ -1738,19 +1749,30 @@ template <typename T>
 cudaError_t build_group_args(csl_batch* B, BatchGroup& G) {
   const int ns = (int)G.sys.size();
   cudaError_t e = cudaSuccess;
+  for (int i = 0; i < ns; ++i)
+    if (!B->plans[G.sys[i]]->ff) G.ff = 0;
+  {
+    const csl_plan* P = G.proto;
+    G.sten_strip = G.ff || P->dim == 2 ? strip_rows(P->dim, P->n[0], P->n[1], P->n[2], (long)kSMs * (G.ff ? 24 : 16) / ns)
+                                       : kStencilStrip;
+    G.sten_blocks = stencil_blocks(P, G.sten_strip);
+  }
   for (int par = 0; par < 2 && e == cudaSuccess; ++par) {
     std::vector<StencilArgs> sa(ns);
     std::vector<RowArgs<T>> p1(ns), p3(ns);
+    std::vector<UpdateArgs> up(ns);
     for (int i = 0; i < ns; ++i) {
       csl_plan* P = B->plans[G.sys[i]];
       StencilArgs a = stencil_args(P, par);
       a.use_cond = 0;
+      a.strip = G.sten_strip;
       sa[i] = a;
-      if (!P->ff) G.ff = 0;
+      up[i] = update_args(P, par);
       p1[i] = p1_args<T>(P, par);
       p3[i] = p3_args<T>(P, par);
     }
     e = upload_array(B, (void**)&G.d_sten[par], sa);
+    if (e == cudaSuccess) e = upload_array(B, (void**)&G.d_upd[par], up);
     if (e == cudaSuccess) e = upload_array(B, &G.d_p1[par], p1);
     if (e == cudaSuccess) e = upload_array(B, &G.d_p3[par], p3);
   }
@@ -1834,9 +1856,8 @@ cudaError_t group_iteration(csl_batch* B, BatchGroup& G, int par, cudaStream_t s
   memset(&sd, 0, sizeof(sd));
   const StencilArgs* sb = (const StencilArgs*)G.d_sten[par];
   const size_t smem = (sizeof(TZ) == 8 && G.ff) ? ff_stencil_smem(P->dim) : 0;
-  cudaError_t e = launch_k(P->use_pdl != 0, stencil_fn<TZ>(P->dim, G.ff != 0, P->vpair != 0), P->sten_blocks * ns, 256,
-                           smem, s,
-                           sd, sb, P->sten_blocks);
+  cudaError_t e = launch_k(P->use_pdl != 0, stencil_fn<TZ>(P->dim, G.ff != 0, P->vpair != 0), G.sten_blocks * ns, 256,
+                           smem, s, sd, sb, G.sten_blocks);
   RowArgs<T> rd;
   memset(&rd, 0, sizeof(rd));
   if (e == cudaSuccess)
@@ -1844,8 +1865,10 @@ cudaError_t group_iteration(csl_batch* B, BatchGroup& G, int par, cudaStream_t s
                       (const RowArgs<T>*)G.d_p1[par], ns);
   if (e == cudaSuccess) e = group_mid_chain<T>(B, G, s, G.d_mid);
   if (e == cudaSuccess)
-    e = launch_row<T>(P->row.N, P->row.wide, LOAD_T, update_store(P), rd, P->row.L, s,
-                      (const RowArgs<T>*)G.d_p3[par], ns);
+    e = launch_row<T>(P->row.N, P->row.wide, LOAD_T, STORE_Z, rd, P->row.L, s, (const RowArgs<T>*)G.d_p3[par], ns);
+  // the update moves the same bytes as fused into the inverse x pass, at the
+  // rate of a streaming kernel
+  if (e == cudaSuccess) e = launch_update<T>(P, par, s, G.d_upd[par], ns);
   return e;
 }
 

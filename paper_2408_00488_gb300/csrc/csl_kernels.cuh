@@ -246,15 +246,16 @@ __host__ __device__ inline long stencil_strips(int dim, int nx, int ny, int nz, 
   return nsx * ((nm + strip - 1) / strip) * (dim == 3 ? ny : 1);
 }
 
-// Strip length for `warps` resident warps on each of the `sms` SMs: 24 for
-// the float-pair stencil (three 8-warp CTAs at 80 registers), 16 for the 2D
-// FP64-arithmetic stencil (two at 128), so that the dependent arithmetic of
-// one warp hides behind the others and every SM gets the same number of
-// strips; 4 .. 64 steps.
-inline int strip_rows(int dim, int nx, int ny, int nz, int sms, int warps) {
+// Strip length for `warps` resident warps: per SM 24 for the float-pair stencil
+// (three 8-warp CTAs at 80 registers), 16 for the 2D FP64-arithmetic stencil
+// (two at 128), so that the dependent arithmetic of one warp hides behind the
+// others and every SM gets the same number of strips; 4 .. 64 steps.  The
+// systems of a batch share the warps: strips as short as a single system's
+// spend a third of their steps filling the operand ring.
+inline int strip_rows(int dim, int nx, int ny, int nz, long warps) {
   const long cols = (long)((nx + 31) / 32) * (dim == 3 ? ny : 1);
   const long nm = dim == 2 ? ny : nz;
-  long per_col = (long)sms * warps / cols;
+  long per_col = warps / cols;
   if (per_col < 1) per_col = 1;
   const long strip = (nm + per_col - 1) / per_col;
   return (int)(strip < 4 ? 4 : strip > 64 ? 64 : strip);
@@ -906,7 +907,11 @@ __device__ __forceinline__ void ff_update(float z, float2 wp, float2 wq, float2 
 }
 
 template <typename TZ, bool VP>
-__global__ void __launch_bounds__(256) k_update(UpdateArgs a) {
+__global__ void __launch_bounds__(256) k_update(UpdateArgs a0, const UpdateArgs* batch, int bps) {
+  const int sys = batch ? (int)(blockIdx.x / bps) : 0;
+  const int bid = batch ? (int)blockIdx.x - sys * bps : (int)blockIdx.x;
+  const int nblk = batch ? bps : (int)gridDim.x;
+  const UpdateArgs a = batch ? batch[sys] : a0;
   if (a.st->done) return;
   const TZ* z = (const TZ*)a.z;
   constexpr int U = kUpdateUnroll;
@@ -915,7 +920,7 @@ __global__ void __launch_bounds__(256) k_update(UpdateArgs a) {
     const float4* wq4 = (const float4*)a.wcur;
     float4* wp4 = (float4*)a.wprev;
     float4* x4 = (float4*)a.x;
-    for (long c0 = (long)blockIdx.x * 256 * U; c0 < a.M; c0 += (long)gridDim.x * 256 * U) {
+    for (long c0 = (long)bid * 256 * U; c0 < a.M; c0 += (long)nblk * 256 * U) {
       float2 zj[U];
       float4 wp[U], wq[U], xo[U];
 #pragma unroll
@@ -944,7 +949,7 @@ __global__ void __launch_bounds__(256) k_update(UpdateArgs a) {
     }
   } else {
     const double wb = a.st->w_b, wc = a.st->w_c, xc = a.st->x_coef;
-    for (long c0 = (long)blockIdx.x * 256 * U; c0 < a.M; c0 += (long)gridDim.x * 256 * U) {
+    for (long c0 = (long)bid * 256 * U; c0 < a.M; c0 += (long)nblk * 256 * U) {
       TZ zj[U];
       double2 wp[U], wq[U], xo[U];
 #pragma unroll
