@@ -1872,6 +1872,113 @@ cudaError_t group_iteration(csl_batch* B, BatchGroup& G, int par, cudaStream_t s
   return e;
 }
 
+// The batched passes' shapes are tuned on the group's own launches: with many
+// systems the CTAs are plenty, and what counts is wide tiles and few
+// instructions, not the latency of one line (n = 511, 64 systems: the shape of
+// a single system's MID pass, one column per CTA, takes 536 us there).  Cached
+// per (pass, number of systems) for the life of the process.
+std::map<std::pair<TuneKey, int>, PassCfg> g_batch_tune_cache;
+
+template <typename T>
+cudaError_t tune_group_pass(csl_batch* B, BatchGroup& G, int kind, void* scratch, cudaEvent_t* ev) {
+  csl_plan* proto = G.proto;
+  PassCfg csl_plan::*field = kind == 0 ? &csl_plan::row : kind == 1 || proto->dim == 2 ? &csl_plan::sy : &csl_plan::sz;
+  const PassCfg keep = proto->*field;
+  if (keep.L.tc || keep.wide >= 3) return cudaSuccess;
+  const int ns = (int)G.sys.size();
+  const std::pair<TuneKey, int> key = {{(int)sizeof(T), kind, keep.N, keep.ncols, keep.nouter}, ns};
+  cudaError_t e = cudaSuccess;
+  PassCfg best = keep;
+  bool hit = false;
+  {
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    auto it = g_batch_tune_cache.find(key);
+    hit = it != g_batch_tune_cache.end() && make_candidate<T>(keep, kind, it->second.wide, it->second.lines, best);
+  }
+  double best_ms = 1e30;
+  for (int w = pass_first_variant<T>(keep.N); w < pass_num_variants(keep.N) && !hit && e == cudaSuccess; ++w) {
+    for (int lines = 1; lines <= 256 && e == cudaSuccess; lines <<= 1) {
+      PassCfg cand;
+      if (!make_candidate<T>(keep, kind, w, lines, cand)) continue;
+      for (int i : G.sys) B->plans[i]->*field = cand;
+      // arguments of the candidate: the x passes P1 and P3, or the strided pass
+      std::vector<RowArgs<T>> ra;
+      std::vector<StridedArgs<T>> sa;
+      for (int i : G.sys) {
+        csl_plan* P = B->plans[i];
+        if (kind == 0) {
+          ra.push_back(p1_args<T>(P, 0));
+        } else {
+          const int ax = kind == 1 || P->dim == 2 ? 1 : 2;
+          sa.push_back(strided_args<T>(P, cand, ax));
+          if (kind == 2) fill_mid<T>(P, sa.back(), ax);
+          sa.back().st = P->st;
+          sa.back().scalar_mode = kind == 2 ? 3 : 0;
+        }
+      }
+      if (kind == 0)
+        for (int i : G.sys) ra.push_back(p3_args<T>(B->plans[i], 0));
+      const void* src = kind == 0 ? (const void*)ra.data() : (const void*)sa.data();
+      e = cudaMemcpyAsync(scratch, src, kind == 0 ? sizeof(ra[0]) * ra.size() : sizeof(sa[0]) * sa.size(),
+                          cudaMemcpyHostToDevice, B->stream);
+      RowArgs<T> rd;
+      StridedArgs<T> sd;
+      memset(&rd, 0, sizeof(rd));
+      memset(&sd, 0, sizeof(sd));
+      double t = 1e30;
+      for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {  // the fastest of three, after one untimed
+        e = cudaEventRecord(ev[0], B->stream);
+        if (kind == 0) {
+          const RowArgs<T>* d = (const RowArgs<T>*)scratch;
+          if (e == cudaSuccess)
+            e = launch_row<T>(cand.N, cand.wide, lanczos_load(proto), STORE_T, rd, cand.L, B->stream, d, ns);
+          if (e == cudaSuccess) e = launch_row<T>(cand.N, cand.wide, LOAD_T, STORE_Z, rd, cand.L, B->stream, d + ns, ns);
+        } else {
+          if (e == cudaSuccess)
+            e = launch_strided<T>(cand.N, cand.wide, kind == 2, sd, cand.L, B->stream, (const StridedArgs<T>*)scratch, ns);
+        }
+        if (e == cudaSuccess) e = cudaEventRecord(ev[1], B->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(B->stream);
+        float ms = 0.f;
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
+        if (rep > 0 && ms < t) t = ms;
+      }
+      if (e == cudaSuccess && t < best_ms) {
+        best_ms = t;
+        best = cand;
+      }
+    }
+  }
+  for (int i : G.sys) B->plans[i]->*field = best;
+  if (e == cudaSuccess && !hit) {
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    g_batch_tune_cache[key] = best;
+  }
+  return e;
+}
+
+template <typename T>
+cudaError_t tune_group(csl_batch* B, BatchGroup& G) {
+  const size_t ns = G.sys.size();
+  void* scratch = nullptr;
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+  cudaError_t e = cudaMalloc(&scratch, ns * (2 * sizeof(RowArgs<T>) > sizeof(StridedArgs<T>) ? 2 * sizeof(RowArgs<T>)
+                                                                                              : sizeof(StridedArgs<T>)));
+  for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreate(&ev[i]);
+  // finite inputs for every pass
+  for (size_t i = 0; i < ns && e == cudaSuccess; ++i) {
+    csl_plan* P = B->plans[G.sys[i]];
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaMemsetAsync(P->v[k], 0, sizeof(double2) * P->M, B->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(P->T, 0, sizeof(typename C2<T>::t) * P->M, B->stream);
+  }
+  for (int kind = 0; kind < 3; ++kind)
+    if (e == cudaSuccess && !(kind == 1 && G.proto->dim == 2)) e = tune_group_pass<T>(B, G, kind, scratch, ev);
+  for (cudaEvent_t x : ev)
+    if (x) cudaEventDestroy(x);
+  if (scratch) cudaFree(scratch);
+  return e;
+}
+
 template <typename T>
 cudaError_t group_prologue(csl_batch* B, BatchGroup& G, cudaStream_t s) {
   csl_plan* P = G.proto;
@@ -2063,6 +2170,7 @@ csl_status csl_batch_create(csl_batch** out, int nsys, const csl_system_desc* sy
     }
     G->sys.push_back(i);
   }
+  const bool fp32 = o.precision != CSL_PREC_FP64;
   for (auto& G : B->groups) {
     // the group shares its prototype's launch shapes
     for (int i : G.sys) {
@@ -2075,8 +2183,9 @@ csl_status csl_batch_create(csl_batch** out, int nsys, const csl_system_desc* sy
     }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&G.branch, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&G.ev, cudaEventDisableTiming);
-    if (e == cudaSuccess)
-      e = o.precision != CSL_PREC_FP64 ? build_group_args<float>(B, G) : build_group_args<double>(B, G);
+    if (e == cudaSuccess && o.autotune && o.lines_per_cta <= 0 && G.sys.size() > 1)
+      e = fp32 ? tune_group<float>(B, G) : tune_group<double>(B, G);
+    if (e == cudaSuccess) e = fp32 ? build_group_args<float>(B, G) : build_group_args<double>(B, G);
   }
   if (e != cudaSuccess) {
     CSL_NOTE(e, "csl_batch_create");
