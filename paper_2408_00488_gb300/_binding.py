@@ -4,6 +4,7 @@ module loads the library and raises if it has not been built."""
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 from dataclasses import dataclass
 from typing import Optional, Sequence, Tuple
@@ -165,9 +166,12 @@ def _torch():
 
 
 def _stream_handle(stream=None) -> int:
+    if stream is not None:
+        return int(stream.cuda_stream)
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    torch.cuda.init()
+    # the handle of torch.cuda.current_stream() without its Stream object (2.9 us a call)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _dptr(t, dtype_names, what: str) -> int:
@@ -228,8 +232,9 @@ class Plan:
         self.warm_start = bool(warm_start)
         self.precision = precision
         h = _P()
+        self._stream = _stream_handle(stream)
         st = lib.csl_plan_create(ctypes.byref(h), dim, n, ptrs, self.lam.real, self.lam.imag,
-                                 ctypes.byref(opt), _stream_handle(stream))
+                                 ctypes.byref(opt), self._stream)
         _check(st, "csl_plan_create")
         self._h = h
         self._faces = None  # the plan keeps its own copy
@@ -253,7 +258,10 @@ class Plan:
         self.close()
 
     def _sync_stream(self, stream=None):
-        lib.csl_plan_set_stream(self._h, _stream_handle(stream))
+        handle = _stream_handle(stream)
+        if handle != self._stream:
+            lib.csl_plan_set_stream(self._h, handle)
+            self._stream = handle
 
     @property
     def gamma(self) -> float:
@@ -273,7 +281,7 @@ class Plan:
         """The library reads and writes whole grid vectors through plain
         pointers, so every tensor passed must hold exactly one grid vector."""
         shape = _grid_vector(t, what) if pairs_ok else tuple(t.shape)
-        if int(np.prod(shape)) != self.M:
+        if math.prod(shape) != self.M:
             raise ValueError(f"{what} must hold one grid vector of {self.M} points (grid {self.shape}), "
                              f"got shape {tuple(t.shape)}")
 
@@ -338,7 +346,7 @@ class Plan:
     def solve_host(self, f_host, z_host, tol: float = 1e-8, maxit: int = 1000) -> Info:
         """Solve with host (CPU, ideally pinned) complex128 tensors/arrays."""
         for t, what in ((f_host, "f_host"), (z_host, "z_host")):
-            if int(np.prod(tuple(t.shape))) != self.M or "complex128" not in str(t.dtype):
+            if math.prod(t.shape) != self.M or "complex128" not in str(t.dtype):
                 raise ValueError(f"{what} must be a complex128 host array of {self.M} points")
         self._sync_stream()
         ci = SolveInfo()
@@ -441,7 +449,7 @@ class Batch:
             raise ValueError(f"one right-hand side (and output) per system: {self.n}")
         for i, shp in enumerate(self.shapes):
             for t in [fs[i]] + ([outs[i]] if outs is not None else []):
-                if int(np.prod(tuple(t.shape))) != int(np.prod(shp)):
+                if math.prod(t.shape) != math.prod(shp):
                     raise ValueError(f"system {i}: a vector of grid {shp} expected, got shape {tuple(t.shape)}")
         zs = [torch.empty_like(f) for f in fs] if outs is None else outs
         fp = (_P * self.n)(*[_dptr(f, ("complex128",), "f") for f in fs])

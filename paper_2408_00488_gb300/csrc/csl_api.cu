@@ -174,7 +174,9 @@ struct csl_plan {
   int body_iters = 2;     // MINRES iterations per WHILE body of the graph
   int upd_blocks = 1;
   std::vector<void*> allocs;
-  size_t bytes = 0;
+  size_t bytes = 0, slab_bytes = 0;
+  char* slab = nullptr;  // csl_plan_create: the rest of the plan's one allocation
+  int slab_pass = 0;
   double *cx = nullptr, *cy = nullptr, *cz = nullptr, *dg = nullptr, *stab = nullptr;
   float2 *cxp = nullptr, *cyp = nullptr, *czp = nullptr;
   float2 alpha2 = {0.f, 0.f};
@@ -211,14 +213,26 @@ struct csl_plan {
 
 namespace {
 
+// Device memory of a plan.  csl_plan_create takes one allocation for nearly all
+// of it (about 25 blocks): it runs through its requests twice, first adding up
+// their sizes (slab_pass 1), then handing out the pieces (2).  0: a block of its
+// own, also for every piece when the single allocation fails.
 void* dalloc(csl_plan* P, size_t bytes, cudaError_t* err) {
   void* p = nullptr;
   if (*err != cudaSuccess) return nullptr;
-  *err = cudaMalloc(&p, bytes ? bytes : 16);
-  if (*err == cudaSuccess) {
-    P->allocs.push_back(p);
-    P->bytes += bytes;
+  const size_t room = ((bytes ? bytes : 16) + 255) / 256 * 256;
+  if (P->slab_pass == 1) {
+    P->slab_bytes += room;
+    return nullptr;
   }
+  P->bytes += bytes;
+  if (P->slab_pass == 2) {
+    p = P->slab;
+    P->slab += room;
+    return p;
+  }
+  *err = cudaMalloc(&p, bytes ? bytes : 16);
+  if (*err == cudaSuccess) P->allocs.push_back(p);
   return p;
 }
 
@@ -787,22 +801,23 @@ int pass_kernels(const csl_plan* P, int kind, int idx[2]) {
   return 1;
 }
 
+// the cached shape of a pass, rebuilt from (variant, lines) for this plan;
+// true also for passes with one shape (tensor-core and long-line variants)
+template <typename T>
+bool tuned_before(PassCfg& c, int kind) {
+  if (c.L.tc || c.wide >= 3) return true;
+  std::lock_guard<std::mutex> lk(g_tune_mu);
+  auto it = g_tune_cache.find({(int)sizeof(T), kind, c.N, c.ncols, c.nouter});
+  PassCfg hit;
+  if (it == g_tune_cache.end() || !make_candidate<T>(c, kind, it->second.wide, it->second.lines, hit)) return false;
+  c = hit;
+  return true;
+}
+
 template <typename T>
 cudaError_t tune_pass(csl_plan* P, PassCfg& c, int kind, cudaEvent_t* ev, const DevState& hst) {
-  if (c.L.tc || c.wide >= 3) return cudaSuccess;  // the tensor-core and long-line variants have one shape
+  if (tuned_before<T>(c, kind)) return cudaSuccess;
   const TuneKey key = {(int)sizeof(T), kind, c.N, c.ncols, c.nouter};
-  {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tune_cache.find(key);
-    if (it != g_tune_cache.end()) {
-      PassCfg hit;
-      // a cached shape is rebuilt from (variant, lines) for this plan's pass
-      if (make_candidate<T>(c, kind, it->second.wide, it->second.lines, hit)) {
-        c = hit;
-        return cudaSuccess;
-      }
-    }
-  }
   int idx[2];
   const int nidx = pass_kernels(P, kind, idx);
   const PassCfg keep = c;
@@ -838,6 +853,9 @@ cudaError_t tune_pass(csl_plan* P, PassCfg& c, int kind, cudaEvent_t* ev, const 
 
 template <typename T>
 cudaError_t autotune(csl_plan* P) {
+  if (tuned_before<T>(P->row, 0) && tuned_before<T>(P->sy, P->dim == 2 ? 2 : 1) &&
+      (P->dim == 2 || tuned_before<T>(P->sz, 2)))
+    return cudaSuccess;
   const DevState h = scratch_state(P);
   DevState* keep = P->st;
   P->st = P->st_prof;
@@ -1097,39 +1115,53 @@ csl_status csl_plan_create(csl_plan** out, int dim, const int64_t n[3], const do
   if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&P->side, cudaStreamNonBlocking);
   if (err == cudaSuccess) err = cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming);
   if (err == cudaSuccess) err = cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming);
-  P->cx = (double*)dalloc(P, nface[0] * 8, &err);
-  P->cy = (double*)dalloc(P, nface[1] * 8, &err);
-  if (dim == 3) P->cz = (double*)dalloc(P, nface[2] * 8, &err);
-  P->dg = (double*)dalloc(P, M * 8, &err);
-  if (o.precision == CSL_PREC_FP64) P->stab = (double*)dalloc(P, M * 8, &err);
-  if (P->vpair && o.float_pair_stencil) {
-    P->cxp = (float2*)dalloc(P, nface[0] * 8, &err);
-    P->cyp = (float2*)dalloc(P, nface[1] * 8, &err);
-    if (dim == 3) P->czp = (float2*)dalloc(P, nface[2] * 8, &err);
+  for (P->slab_pass = 1; P->slab_pass <= 2 && err == cudaSuccess; ++P->slab_pass) {
+    if (P->slab_pass == 2) {
+      void* p = nullptr;
+      if (cudaMalloc(&p, P->slab_bytes) == cudaSuccess) {
+        P->allocs.push_back(p);
+        P->slab = (char*)p;
+      } else {  // piece by piece
+        (void)cudaGetLastError();
+        P->slab_pass = 0;
+      }
+    }
+    P->cx = (double*)dalloc(P, nface[0] * 8, &err);
+    P->cy = (double*)dalloc(P, nface[1] * 8, &err);
+    if (dim == 3) P->cz = (double*)dalloc(P, nface[2] * 8, &err);
+    P->dg = (double*)dalloc(P, M * 8, &err);
+    if (o.precision == CSL_PREC_FP64) P->stab = (double*)dalloc(P, M * 8, &err);
+    if (P->vpair && o.float_pair_stencil) {
+      P->cxp = (float2*)dalloc(P, nface[0] * 8, &err);
+      P->cyp = (float2*)dalloc(P, nface[1] * 8, &err);
+      if (dim == 3) P->czp = (float2*)dalloc(P, nface[2] * 8, &err);
+    }
+    for (int d = 0; d < dim; ++d) {
+      const int N = P->n[d] + 1;
+      P->mu_d[d] = (double*)dalloc(P, (size_t)P->n[d] * 8, &err);
+      P->mu_f[d] = (float*)dalloc(P, (size_t)P->n[d] * 4, &err);
+      P->tw[d] = dalloc(P, (size_t)(N / 2) * 2 * tsz, &err);
+      P->hs[d] = dalloc(P, (size_t)(N / 2 + 1) * tsz, &err);
+      P->tp[d] = dalloc(P, (size_t)((fp64 ? pass_tp_total<double>(N) : pass_tp_total<float>(N)) + 1) * 2 * tsz, &err);
+    }
+    P->b = (double2*)dalloc(P, M * 16, &err);
+    P->x = (double2*)dalloc(P, M * 16, &err);
+    P->io = (double2*)dalloc(P, M * 16, &err);
+    if (P->warm) P->x0 = (double2*)dalloc(P, M * 16, &err);
+    if (P->hist_cap > 0) P->hist = (double*)dalloc(P, (size_t)P->hist_cap * 8, &err);
+    for (int i = 0; i < 2; ++i) {
+      P->v[i] = (double2*)dalloc(P, M * 16, &err);
+      P->w[i] = (double2*)dalloc(P, M * 16, &err);
+      P->z[i] = dalloc(P, M * 2 * tsz, &err);
+    }
+    P->T = dalloc(P, M * 2 * tsz, &err);
+    P->st = (DevState*)dalloc(P, sizeof(DevState), &err);
+    P->st_prof = (DevState*)dalloc(P, sizeof(DevState), &err);
+    P->partials = (double*)dalloc(P, (size_t)kMaxRedBlocks * 4 * 8, &err);
+    P->u64 = (unsigned long long*)dalloc(P, 8 * 8, &err);
+    if (P->slab_pass == 0) break;
   }
-  for (int d = 0; d < dim; ++d) {
-    const int N = P->n[d] + 1;
-    P->mu_d[d] = (double*)dalloc(P, (size_t)P->n[d] * 8, &err);
-    P->mu_f[d] = (float*)dalloc(P, (size_t)P->n[d] * 4, &err);
-    P->tw[d] = dalloc(P, (size_t)(N / 2) * 2 * tsz, &err);
-    P->hs[d] = dalloc(P, (size_t)(N / 2 + 1) * tsz, &err);
-    P->tp[d] = dalloc(P, (size_t)((fp64 ? pass_tp_total<double>(N) : pass_tp_total<float>(N)) + 1) * 2 * tsz, &err);
-  }
-  P->b = (double2*)dalloc(P, M * 16, &err);
-  P->x = (double2*)dalloc(P, M * 16, &err);
-  P->io = (double2*)dalloc(P, M * 16, &err);
-  if (P->warm) P->x0 = (double2*)dalloc(P, M * 16, &err);
-  if (P->hist_cap > 0) P->hist = (double*)dalloc(P, (size_t)P->hist_cap * 8, &err);
-  for (int i = 0; i < 2; ++i) {
-    P->v[i] = (double2*)dalloc(P, M * 16, &err);
-    P->w[i] = (double2*)dalloc(P, M * 16, &err);
-    P->z[i] = dalloc(P, M * 2 * tsz, &err);
-  }
-  P->T = dalloc(P, M * 2 * tsz, &err);
-  P->st = (DevState*)dalloc(P, sizeof(DevState), &err);
-  P->st_prof = (DevState*)dalloc(P, sizeof(DevState), &err);
-  P->partials = (double*)dalloc(P, (size_t)kMaxRedBlocks * 4 * 8, &err);
-  P->u64 = (unsigned long long*)dalloc(P, 8 * 8, &err);
+  P->slab_pass = 0;
   if (err != cudaSuccess) {
     CSL_NOTE(err, "device allocation");
     (void)cudaGetLastError();
@@ -1145,36 +1177,31 @@ csl_status csl_plan_create(csl_plan** out, int dim, const int64_t n[3], const do
 
   // coefficient faces: a_e / h^2, min / max / validity (Eq. 1 and Eq. 4's a_min, a_max)
   {
-    unsigned long long init[3] = {~0ull, 0ull, 0ull};
+    const unsigned long long init[3] = {~0ull, 0ull, 0ull};
     double* dst[3] = {P->cx, P->cy, P->cz};
-    double amin = INFINITY, amax = 0.0;
-    for (int d = 0; d < dim; ++d) {
-      err = cudaMemcpyAsync(P->u64, init, sizeof(init), cudaMemcpyHostToDevice, s);
-      if (err == cudaSuccess) {
-        const long cnt = nface[d];
-        const int blocks = (int)((cnt + 255) / 256 < 1024 ? (cnt + 255) / 256 : 1024);
-        k_scale_faces<<<blocks, 256, 0, s>>>(coef_faces[d], dst[d], cnt, 1.0 / (P->h[d] * P->h[d]), P->u64);
-        err = cudaGetLastError();
-      }
-      unsigned long long res[3] = {0, 0, 0};
-      if (err == cudaSuccess) err = cudaMemcpyAsync(res, P->u64, sizeof(res), cudaMemcpyDeviceToHost, s);
-      if (err == cudaSuccess) err = cudaStreamSynchronize(s);
-      if (err != cudaSuccess) {
-        CSL_NOTE(err, "coefficient set-up");
-        (void)cudaGetLastError();
-        free_plan(P);
-        return CSL_CUDA_ERROR;
-      }
-      if (res[2]) {
-        free_plan(P);
-        return CSL_INVALID_ARG;
-      }
-      double lo, hi;
-      memcpy(&lo, &res[0], 8);
-      memcpy(&hi, &res[1], 8);
-      amin = lo < amin ? lo : amin;
-      amax = hi > amax ? hi : amax;
+    unsigned long long res[3] = {0, 0, 0};
+    err = cudaMemcpyAsync(P->u64, init, sizeof(init), cudaMemcpyHostToDevice, s);
+    for (int d = 0; d < dim && err == cudaSuccess; ++d) {
+      const long cnt = nface[d];
+      const int blocks = (int)((cnt + 255) / 256 < 1024 ? (cnt + 255) / 256 : 1024);
+      k_scale_faces<<<blocks, 256, 0, s>>>(coef_faces[d], dst[d], cnt, 1.0 / (P->h[d] * P->h[d]), P->u64);
+      err = cudaGetLastError();
     }
+    if (err == cudaSuccess) err = cudaMemcpyAsync(res, P->u64, sizeof(res), cudaMemcpyDeviceToHost, s);
+    if (err == cudaSuccess) err = cudaStreamSynchronize(s);
+    if (err != cudaSuccess) {
+      CSL_NOTE(err, "coefficient set-up");
+      (void)cudaGetLastError();
+      free_plan(P);
+      return CSL_CUDA_ERROR;
+    }
+    if (res[2]) {
+      free_plan(P);
+      return CSL_INVALID_ARG;
+    }
+    double amin, amax;
+    memcpy(&amin, &res[0], 8);
+    memcpy(&amax, &res[1], 8);
     P->amin = amin;
     P->amax = amax;
     P->gamma = (o.gamma_override > 0.0 && isfinite(o.gamma_override)) ? o.gamma_override : sqrt(amin * amax);

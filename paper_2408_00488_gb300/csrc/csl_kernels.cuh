@@ -1125,6 +1125,23 @@ static __global__ void k_x_out_add(const double2* __restrict__ d, int pairs, con
 // ---------------------------------------------------------------------------
 // Plan set-up kernels
 // ---------------------------------------------------------------------------
+// min and max of the threads' values into minmax[0], [1], one atomic per warp
+// (one per thread, up to half a million on one address, took longer than the
+// rest of the kernel)
+__device__ __forceinline__ void warp_minmax(unsigned long long* minmax, unsigned long long lmin,
+                                            unsigned long long lmax) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long a = __shfl_xor_sync(0xffffffffu, lmin, o), b = __shfl_xor_sync(0xffffffffu, lmax, o);
+    lmin = a < lmin ? a : lmin;
+    lmax = b > lmax ? b : lmax;
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&minmax[0], lmin);
+    atomicMax(&minmax[1], lmax);
+  }
+}
+
 // scaled copy of one face array (a_e / h^2) and its min / max / validity
 static __global__ void k_scale_faces(const double* __restrict__ src, double* __restrict__ dst, long count,
                               double inv_h2, unsigned long long* minmax /* [min bits, max bits, bad] */) {
@@ -1139,8 +1156,7 @@ static __global__ void k_scale_faces(const double* __restrict__ src, double* __r
     }
     dst[i] = v * inv_h2;
   }
-  atomicMin(&minmax[0], lmin);
-  atomicMax(&minmax[1], lmax);
+  warp_minmax(minmax, lmin, lmax);
   if (bad) atomicOr(&minmax[2], 1ull);
 }
 
@@ -1190,8 +1206,7 @@ __global__ void k_scale_table(Grid g, const double* mux, const double* muy, cons
     lmin = bits < lmin ? bits : lmin;
     lmax = bits > lmax ? bits : lmax;
   }
-  atomicMin(&qminmax[0], lmin);
-  atomicMax(&qminmax[1], lmax);
+  warp_minmax(qminmax, lmin, lmax);
 }
 
 // dL/da_e = -h^{-2} Re(conj(dy) dz) over the faces of one axis (unscaled a_e)
