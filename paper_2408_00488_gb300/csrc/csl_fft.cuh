@@ -624,8 +624,10 @@ struct LineDst<T, N, 3> {
 // The FP64 form: 64-bit block fixed point (csl_fix.cuh).  The line buffer
 // holds doubles before and after; input and output positions agree.  Tables:
 // half sines and pass tables (signed digits, the sizes of a double and a
-// double2), in shared memory up to N = 1024.
-template <int N, int LANES, bool GLOBAL>
+// double2), read through the L1: copied into each CTA's shared memory (22 KB at
+// N = 1024), they kept CTAs of one line from filling the SM (x pass at n = 1023
+// 34.6 -> 26.8 us, at 3D n = 127 with the Lanczos step 55.2 -> 47.6).
+template <int N, int LANES>
 struct FixDst {
   typedef FixLine<N, LANES> F;
   enum { TPL = LANES, LS = fix_line_stride<N>(), SCRATCH = 2 * (LANES / 32 > 4 ? LANES / 32 : 4) };
@@ -634,17 +636,9 @@ struct FixDst {
     const fxw* tp;
   };
   struct Tables {
-    static constexpr int kTpN = fix_table_entries<N, LANES>();
-    static constexpr size_t kTp = (((size_t)(N / 2 + 1) * 8 + 15) / 16) * 16,
-                            kBytes = GLOBAL ? 0 : kTp + (size_t)kTpN * sizeof(fxw);
-    static __device__ __forceinline__ Tab load(unsigned char* smem, const double2*, const double* hs,
-                                               const double2* tp) {
-      if constexpr (GLOBAL) return {(const int2*)hs, (const fxw*)tp};
-      int2* s_hs = (int2*)smem;
-      fxw* s_tp = (fxw*)(smem + kTp);
-      for (int i = threadIdx.x; i <= N / 2; i += blockDim.x) s_hs[i] = ((const int2*)hs)[i];
-      for (int i = threadIdx.x; i < kTpN; i += blockDim.x) s_tp[i] = ((const fxw*)tp)[i];
-      return {s_hs, s_tp};
+    static constexpr size_t kBytes = 0;
+    static __device__ __forceinline__ Tab load(unsigned char*, const double2*, const double* hs, const double2* tp) {
+      return {(const int2*)hs, (const fxw*)tp};
     }
   };
   static __device__ __forceinline__ int in_pos(int j) { return fpad(j); }
@@ -666,11 +660,11 @@ struct FixDst {
 // lanes per line: 8 to 16 values a lane; N = 512 and 1024 have no
 // warp-per-line variant (32 values a lane spill), 0 stands for 1 there
 template <int N>
-struct LineDst<double, N, 0> : FixDst<N, N == 32 ? 4 : N >= 512 ? 64 : DstShape<N>::TPL, false> {};
+struct LineDst<double, N, 0> : FixDst<N, N == 32 ? 4 : N >= 512 ? 64 : DstShape<N>::TPL> {};
 template <int N, int V>
-struct LineDst<double, N, V> : FixDst<N, wide_tpl(V), false> {};
+struct LineDst<double, N, V> : FixDst<N, wide_tpl(V)> {};
 template <int N>
-struct LineDst<double, N, 3> : FixDst<N, BigShape<N>::TPL, true> {};
+struct LineDst<double, N, 3> : FixDst<N, BigShape<N>::TPL> {};
 
 // Host-side size of the extra twiddle table of length N in the FP32 forms.
 __host__ __device__ constexpr int line_tp_size(int N, int wide) {
