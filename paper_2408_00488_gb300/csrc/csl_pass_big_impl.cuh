@@ -16,29 +16,17 @@ cudaError_t launch_row_big_n(int load, int store, const RowArgs<T>& a, const Pas
     if (load == LOAD_LANCZOS_V64) load = LOAD_LANCZOS;
     if (store == STORE_Z_UPDATE_V64) store = STORE_Z_UPDATE;
   }
+  auto go = [&](auto k) { return launch_k(L.pdl != 0, k, grid, L.threads, L.smem, s, a, batch, bps); };
   if constexpr (sizeof(T) == 4) {  // FP32 transform, FP64 vectors
-    if (load == LOAD_LANCZOS_V64 && store == STORE_T) {
-      k_row<T, N, 3, LOAD_LANCZOS_V64, STORE_T><<<grid, L.threads, L.smem, s>>>(a, batch, bps);
-      return cudaGetLastError();
-    }
-    if (load == LOAD_T && store == STORE_Z_UPDATE_V64) {
-      k_row<T, N, 3, LOAD_T, STORE_Z_UPDATE_V64><<<grid, L.threads, L.smem, s>>>(a, batch, bps);
-      return cudaGetLastError();
-    }
+    if (load == LOAD_LANCZOS_V64 && store == STORE_T) return go(k_row<T, N, 3, LOAD_LANCZOS_V64, STORE_T>);
+    if (load == LOAD_T && store == STORE_Z_UPDATE_V64) return go(k_row<T, N, 3, LOAD_T, STORE_Z_UPDATE_V64>);
   }
-  if (load == LOAD_V && store == STORE_T)
-    k_row<T, N, 3, LOAD_V, STORE_T><<<grid, L.threads, L.smem, s>>>(a, batch, bps);
-  else if (load == LOAD_LANCZOS && store == STORE_T)
-    k_row<T, N, 3, LOAD_LANCZOS, STORE_T><<<grid, L.threads, L.smem, s>>>(a, batch, bps);
-  else if (load == LOAD_T && store == STORE_Z)
-    k_row<T, N, 3, LOAD_T, STORE_Z><<<grid, L.threads, L.smem, s>>>(a, batch, bps);
-  else if (load == LOAD_T && store == STORE_Z_UPDATE)
-    k_row<T, N, 3, LOAD_T, STORE_Z_UPDATE><<<grid, L.threads, L.smem, s>>>(a, batch, bps);
-  else if (load == LOAD_T && store == STORE_D)
-    k_row<T, N, 3, LOAD_T, STORE_D><<<grid, L.threads, L.smem, s>>>(a, batch, bps);
-  else
-    return cudaErrorInvalidValue;
-  return cudaGetLastError();
+  if (load == LOAD_V && store == STORE_T) return go(k_row<T, N, 3, LOAD_V, STORE_T>);
+  if (load == LOAD_LANCZOS && store == STORE_T) return go(k_row<T, N, 3, LOAD_LANCZOS, STORE_T>);
+  if (load == LOAD_T && store == STORE_Z) return go(k_row<T, N, 3, LOAD_T, STORE_Z>);
+  if (load == LOAD_T && store == STORE_Z_UPDATE) return go(k_row<T, N, 3, LOAD_T, STORE_Z_UPDATE>);
+  if (load == LOAD_T && store == STORE_D) return go(k_row<T, N, 3, LOAD_T, STORE_D>);
+  return cudaErrorInvalidValue;
 }
 
 template <typename T>
@@ -74,12 +62,9 @@ cudaError_t launch_strided_big(int N, bool mid, const StridedArgs<T>& a, const P
   const int grid = batch ? L.blocks * nsys : L.blocks;
   switch (N) {
 #define CASE(NN)                                                                              \
-  case NN:                                                                                    \
-    if (mid)                                                                                  \
-      k_strided<T, NN, 3, true><<<grid, L.threads, L.smem, s>>>(a, batch, L.blocks);          \
-    else                                                                                      \
-      k_strided<T, NN, 3, false><<<grid, L.threads, L.smem, s>>>(a, batch, L.blocks);         \
-    return cudaGetLastError();
+  case NN:                                                                                               \
+    return mid ? launch_k(L.pdl != 0, k_strided<T, NN, 3, true>, grid, L.threads, L.smem, s, a, batch, L.blocks) \
+               : launch_k(L.pdl != 0, k_strided<T, NN, 3, false>, grid, L.threads, L.smem, s, a, batch, L.blocks);
     CSL_FOR_EACH_BIG_N(CASE)
 #undef CASE
   }

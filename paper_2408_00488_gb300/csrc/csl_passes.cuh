@@ -20,8 +20,9 @@
 #include <vector>
 
 // two CTAs of 256 threads per SM (at most 128 registers per thread), three
-// with 128 lanes per line in FP32; one of a long line's
-#define CSL_PASS_MINB(T, V) ((V) < 3 ? (sizeof(T) == 4 && (V) == 2 ? 3 : 2) : 1)
+// with 128 lanes per line in FP32; one of a line of 8192's 512 lanes.  Without
+// the bound the long lines took 160 to 255 registers, one CTA of 8 warps per SM.
+#define CSL_PASS_MINB(T, N, V) ((V) < 3 ? (sizeof(T) == 4 && (V) == 2 ? 3 : 2) : (N) < 8192 ? 2 : 1)
 // The warp-per-line row passes of length 1024 that stream MINRES vectors
 // from HBM (the Lanczos step before the forward transform, the w/x update
 // after the inverse one) keep many loads in flight per lane, so they take the
@@ -30,7 +31,7 @@
 #define CSL_ROW_STREAMS(T, N, V, LOAD_MODE, STORE_MODE) \
   (sizeof(T) == 4 && (N) == 1024 && (V) == 0 && ((LOAD_MODE) >= 2 || (STORE_MODE) >= 3))
 #define CSL_ROW_MINB(T, N, V, LOAD_MODE, STORE_MODE) \
-  (CSL_ROW_STREAMS(T, N, V, LOAD_MODE, STORE_MODE) ? 1 : CSL_PASS_MINB(T, V))
+  (CSL_ROW_STREAMS(T, N, V, LOAD_MODE, STORE_MODE) ? 1 : CSL_PASS_MINB(T, N, V))
 
 namespace csl {
 
@@ -375,7 +376,7 @@ struct MidScale {
 };
 
 template <typename T, int N, int WIDE, bool MID>
-__global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_PASS_MINB(T, WIDE)) k_strided(StridedArgs<T> a0, const StridedArgs<T>* batch, int bps) {
+__global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_PASS_MINB(T, N, WIDE)) k_strided(StridedArgs<T> a0, const StridedArgs<T>* batch, int bps) {
   typedef typename C2<T>::t c_t;
   typedef LineDst<T, N, WIDE> D;
   const int sys = batch ? (int)(blockIdx.x / bps) : 0;
