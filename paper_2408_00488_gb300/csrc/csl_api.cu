@@ -202,7 +202,7 @@ struct csl_plan {
   unsigned long long* u64 = nullptr;
   PassCfg row, sy, sz;
   int sten_blocks = 1, ew_blocks = 1;
-  int sten_strip = kStencilStrip;  // steps per warp strip of the stencil
+  int sten_strip = 1;  // steps per warp strip of the stencil
   double cnorm = 1;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
@@ -1236,8 +1236,7 @@ csl_status csl_plan_create(csl_plan** out, int dim, const int64_t n[3], const do
     }
   }
   {
-    P->sten_strip = P->ff ? strip_rows(dim, nx, ny, nz, kSMs * 24)
-                    : dim == 2 ? strip_rows(dim, nx, ny, nz, kSMs * 16) : kStencilStrip;
+    P->sten_strip = strip_rows(dim, nx, ny, nz, kSMs * stencil_warps(dim, P->ff != 0));
     P->sten_blocks = stencil_blocks(P, P->sten_strip);
   }
   Grid g;
@@ -1780,8 +1779,7 @@ cudaError_t build_group_args(csl_batch* B, BatchGroup& G) {
     if (!B->plans[G.sys[i]]->ff) G.ff = 0;
   {
     const csl_plan* P = G.proto;
-    G.sten_strip = G.ff || P->dim == 2 ? strip_rows(P->dim, P->n[0], P->n[1], P->n[2], (long)kSMs * (G.ff ? 24 : 16) / ns)
-                                       : kStencilStrip;
+    G.sten_strip = strip_rows(P->dim, P->n[0], P->n[1], P->n[2], (long)kSMs * stencil_warps(P->dim, G.ff != 0) / ns);
     G.sten_blocks = stencil_blocks(P, G.sten_strip);
   }
   for (int par = 0; par < 2 && e == cudaSuccess; ++par) {

@@ -226,10 +226,6 @@ __device__ __forceinline__ float2 shfl_down_f2(float2 v) {
   return make_float2(__shfl_down_sync(0xffffffffu, v.x, 1), __shfl_down_sync(0xffffffffu, v.y, 1));
 }
 
-// Planes one warp walks per strip of the 3D FP64-arithmetic stencil; the
-// float-pair stencil and the 2D FP64 one size their strips per plan
-// (strip_rows).
-constexpr int kStencilStrip = 16;
 
 __device__ __forceinline__ double2 shfl_up_d2(double2 v) {
   return make_double2(__shfl_up_sync(0xffffffffu, v.x, 1), __shfl_up_sync(0xffffffffu, v.y, 1));
@@ -246,20 +242,28 @@ __host__ __device__ inline long stencil_strips(int dim, int nx, int ny, int nz, 
   return nsx * ((nm + strip - 1) / strip) * (dim == 3 ? ny : 1);
 }
 
-// Strip length for `warps` resident warps: per SM 24 for the float-pair stencil
-// (three 8-warp CTAs at 80 registers), 16 for the 2D FP64-arithmetic stencil
-// (two at 128), so that the dependent arithmetic of one warp hides behind the
-// others and every SM gets the same number of strips; 4 .. 64 steps.  The
-// systems of a batch share the warps: strips as short as a single system's
-// spend a third of their steps filling the operand ring.
+// Strip length for `warps` resident warps (stencil_warps per SM; the systems of
+// a batch share them): the fewest steps of the longest-running warp, i.e. the
+// waves of warps times a strip's steps and the two it takes to fill the operand
+// ring.  n = 63: strips of one step, 9.9 us, where strips of four took 13.9.  3D, n = 127, float pairs: strips of 19 planes gave 3556 warps to 2432
+// places, two waves of 21 steps; strips of 32 give one of 34.
 inline int strip_rows(int dim, int nx, int ny, int nz, long warps) {
   const long cols = (long)((nx + 31) / 32) * (dim == 3 ? ny : 1);
   const long nm = dim == 2 ? ny : nz;
-  long per_col = warps / cols;
-  if (per_col < 1) per_col = 1;
-  const long strip = (nm + per_col - 1) / per_col;
-  return (int)(strip < 4 ? 4 : strip > 64 ? 64 : strip);
+  long best = nm, cost = -1;
+  for (long strip = 1; strip <= nm; ++strip) {
+    const long strips = cols * ((nm + strip - 1) / strip);
+    const long c = ((strips + warps - 1) / (warps > 0 ? warps : 1)) * (strip + 2);
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = strip;
+    }
+  }
+  return (int)best;
 }
+// resident warps of the stencil per SM: three CTAs of 8 warps for the 2D
+// float-pair kernel (80 registers), two for the others (128)
+inline int stencil_warps(int dim, bool ff) { return ff && dim == 2 ? 24 : 16; }
 
 // One value of a strip and its marching window: m-1, m, m+1 along the strip,
 // x-1 / x+1 by warp shuffles (the strip's edge lanes load theirs), and in 3D
