@@ -126,7 +126,7 @@ void make_fix_tables(int N, std::vector<int2>& hs, std::vector<fxw>& tp) {
     hs[j] = make_int2(d.h, d.l);
   }
   tp.clear();
-  for (int v = 0; v <= (N == 512 || N == 1024 ? 2 : 0); v += 2) {
+  for (int v = 0; v >= 0; v = v == 0 ? fix_second_table(N) : -1) {  // in the order of pass_tp_offset
     const FixRadices f = fix_radices_of(N, v);
     int ls = f.r[0];
     for (int p = 1; p < f.np; ++p) {
@@ -762,7 +762,7 @@ std::mutex g_tune_mu;
 // loader, so a shape read from a file is rebuilt and checked the same way.
 template <typename T>
 bool make_candidate(const PassCfg& c, int kind, int w, int lines, PassCfg& cand) {
-  if (w < 0 || w >= pass_num_variants(c.N) || lines < 1 || (lines & (lines - 1))) return false;
+  if (w < 0 || w >= pass_num_variants<T>(c.N) || lines < 1 || (lines & (lines - 1))) return false;
   const int tpl = pass_tpl<T>(c.N, w);
   if (lines * tpl < 32 || lines * tpl > 256) return false;
   cand = c;
@@ -825,7 +825,7 @@ cudaError_t tune_pass(csl_plan* P, PassCfg& c, int kind, cudaEvent_t* ev, const 
   double best_ms = 1e30;
   double ms[8];
   cudaError_t e = cudaSuccess;
-  for (int w = pass_first_variant<T>(keep.N); w < pass_num_variants(keep.N) && e == cudaSuccess; ++w) {
+  for (int w = pass_first_variant<T>(keep.N); w < pass_num_variants<T>(keep.N) && e == cudaSuccess; ++w) {
     for (int lines = 1; lines <= 256 && e == cudaSuccess; lines <<= 1) {
       PassCfg cand;
       if (!make_candidate<T>(keep, kind, w, lines, cand)) continue;
@@ -893,7 +893,7 @@ bool tune_entry_valid(const TuneKey& k, int wide, int lines) {
   if (k.kind < 0 || k.kind > 2) return false;
   if (k.N < 4 || k.N > 1024 || ilog2_exact(k.N) < 0) return false;
   if (k.ncols < 1 || k.nouter < 1) return false;
-  if (wide < 0 || wide >= pass_num_variants(k.N)) return false;
+  if (wide < 0 || wide >= (k.prec == 8 ? pass_num_variants<double>(k.N) : pass_num_variants<float>(k.N))) return false;
   return lines >= 1 && lines <= 256 && !(lines & (lines - 1));
 }
 
@@ -1921,7 +1921,7 @@ cudaError_t tune_group_pass(csl_batch* B, BatchGroup& G, int kind, void* scratch
     hit = it != g_batch_tune_cache.end() && make_candidate<T>(keep, kind, it->second.wide, it->second.lines, best);
   }
   double best_ms = 1e30;
-  for (int w = pass_first_variant<T>(keep.N); w < pass_num_variants(keep.N) && !hit && e == cudaSuccess; ++w) {
+  for (int w = pass_first_variant<T>(keep.N); w < pass_num_variants<T>(keep.N) && !hit && e == cudaSuccess; ++w) {
     for (int lines = 1; lines <= 256 && e == cudaSuccess; lines <<= 1) {
       PassCfg cand;
       if (!make_candidate<T>(keep, kind, w, lines, cand)) continue;

@@ -657,14 +657,12 @@ struct FixDst {
     if constexpr (LANES > 1) fx_line_sync(LANES);
   }
 };
-// lanes per line: 8 to 16 values a lane; N = 512 and 1024 have no
-// warp-per-line variant (32 values a lane spill), 0 stands for 1 there
 template <int N>
-struct LineDst<double, N, 0> : FixDst<N, N == 32 ? 4 : N >= 512 ? 64 : DstShape<N>::TPL> {};
+struct LineDst<double, N, 0> : FixDst<N, fix_lanes(N, 0)> {};
 template <int N, int V>
-struct LineDst<double, N, V> : FixDst<N, wide_tpl(V)> {};
+struct LineDst<double, N, V> : FixDst<N, fix_lanes(N, V)> {};
 template <int N>
-struct LineDst<double, N, 3> : FixDst<N, BigShape<N>::TPL> {};
+struct LineDst<double, N, 3> : FixDst<N, fix_lanes(N, 3)> {};
 
 // Host-side size of the extra twiddle table of length N in the FP32 forms.
 __host__ __device__ constexpr int line_tp_size(int N, int wide) {

@@ -312,15 +312,28 @@ __device__ __forceinline__ double fx_to_double(long long v, int q) {
 }
 
 // ---- shapes ----------------------------------------------------------------------
-// Radices per length and lanes per line.  The first radix is the largest (its
-// products round at the finest scale), and a lane holds N / TPL values; the
-// following radices are at most 8 where that keeps every shift <= kFxMaxShift
+// Lanes per line and radices.  One lane's values are a long serial chain on few
+// warps, so a line takes as many lanes as leave each 4 to 8 values (16 at most):
+// n = 63, 16 lanes instead of 8, iteration 48.8 -> 34.6 us; n = 127, 32 instead
+// of 8, 77.8 -> 30.9; n = 31, 8 instead of 4, 48 -> 34.5.  N = 128 and 256 have
+// two variants: with many lines, as in 3D, fewer lanes and passes win (n = 127
+// in 3D 357 us with 16 lanes, 370 with 32, 384 with 8).  N = 512 and 1024: 64
+// lanes (variant 1, and 0, which has no kernels of its own) or 128 (variant 2).
+// The first radix is the largest (its products round at the finest scale); the
+// following ones are at most 8 where that keeps every shift <= kFxMaxShift
 // without giving up bits of S1.
+__host__ __device__ constexpr int fix_lanes(int N, int variant) {
+  return N <= 8 ? 1 : N == 16 ? 4 : N == 32 ? 8 : N == 64 ? 16 : N == 128 ? (variant ? 32 : 16)
+         : N == 256 ? (variant ? 64 : 32) : N <= 1024 ? (variant == 2 ? 128 : 64) : N <= 4096 ? 256 : 512;
+}
 template <int N, int TPL> struct FixShape;
-template <> struct FixShape<32, 4> { enum { NP = 2, R0 = 8, R1 = 4, R2 = 1, R3 = 1 }; };
-template <> struct FixShape<64, 8> { enum { NP = 2, R0 = 8, R1 = 8, R2 = 1, R3 = 1 }; };
-template <> struct FixShape<128, 8> { enum { NP = 2, R0 = 16, R1 = 8, R2 = 1, R3 = 1 }; };
-template <> struct FixShape<256, 16> { enum { NP = 2, R0 = 16, R1 = 16, R2 = 1, R3 = 1 }; };
+template <> struct FixShape<16, 4> { enum { NP = 2, R0 = 4, R1 = 4, R2 = 1, R3 = 1 }; };
+template <> struct FixShape<32, 8> { enum { NP = 3, R0 = 4, R1 = 4, R2 = 2, R3 = 1 }; };
+template <> struct FixShape<64, 16> { enum { NP = 3, R0 = 4, R1 = 4, R2 = 4, R3 = 1 }; };
+template <> struct FixShape<128, 16> { enum { NP = 3, R0 = 8, R1 = 4, R2 = 4, R3 = 1 }; };
+template <> struct FixShape<128, 32> { enum { NP = 3, R0 = 8, R1 = 4, R2 = 4, R3 = 1 }; };
+template <> struct FixShape<256, 32> { enum { NP = 3, R0 = 8, R1 = 8, R2 = 4, R3 = 1 }; };
+template <> struct FixShape<256, 64> { enum { NP = 4, R0 = 4, R1 = 4, R2 = 4, R3 = 4 }; };
 template <> struct FixShape<512, 64> { enum { NP = 3, R0 = 8, R1 = 8, R2 = 8, R3 = 1 }; };
 template <> struct FixShape<512, 128> { enum { NP = 4, R0 = 8, R1 = 4, R2 = 4, R3 = 4 }; };
 template <> struct FixShape<1024, 64> { enum { NP = 3, R0 = 16, R1 = 8, R2 = 8, R3 = 1 }; };
@@ -589,7 +602,7 @@ struct FixLine {
   }
 };
 
-// lines of N <= 16 points: the whole line in one lane's registers
+// lines of 4 or 8 points: the whole line in one lane's registers
 template <int N>
 struct FixLine<N, 1> {
   enum { S1 = 61 - fx_log2(N) };
@@ -650,15 +663,6 @@ struct FixLine<N, 1> {
 template <int N>
 __host__ __device__ constexpr int fix_line_stride() {
   return N <= 256 ? fpad(N) | 1 : ((fpad(N) + 7) / 8) * 8 + 2;
-}
-
-// pass-table entries of (N, TPL); 0 when the line stays in one lane
-template <int N, int TPL>
-__host__ __device__ constexpr int fix_table_entries() {
-  if constexpr (TPL == 1)
-    return 0;
-  else
-    return fix_tp_entries<FixShape<N, TPL>>();
 }
 
 // Pass table of the radices r[0 .. np-1], host or device: entry e of pass p is

@@ -1,7 +1,7 @@
-// FP64 instantiation of the sine-transform passes, N = 128 and 256.
+// FP64 instantiation of the sine-transform passes, N = 128.
 #include "csl_pass_impl.cuh"
 
 namespace csl {
 CSL_INSTANTIATE_PASS(double, 128, 0)
-CSL_INSTANTIATE_PASS(double, 256, 0)
+CSL_INSTANTIATE_PASS(double, 128, 1)
 }  // namespace csl

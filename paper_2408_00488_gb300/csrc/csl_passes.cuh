@@ -502,10 +502,14 @@ struct PassLaunch {
 #define CSL_FOR_EACH_N(X) X(4) X(8) X(16) X(32) X(64) X(128) X(256) X(512) X(1024)
 
 // N = 512 and 1024 exist in three variants (warp per line, 64 and 128 lanes
-// per line: wide = 0, 1, 2); the autotuner picks one per pass.
+// per line: wide = 0, 1, 2; in FP64 0 stands for 1), N = 128 and 256 in two in
+// FP64 (fix_lanes); the autotuner picks one per pass.
 inline bool pass_has_wide(int N) { return N == 512 || N == 1024; }
-inline int pass_num_variants(int N) { return pass_has_wide(N) ? 3 : 1; }
-// the first variant the tuner tries: the FP64 form's variant 0 is its 1
+template <typename T>
+inline int pass_num_variants(int N) {
+  return pass_has_wide(N) ? 3 : sizeof(T) == 8 && (N == 128 || N == 256) ? 2 : 1;
+}
+// the first variant the tuner tries
 template <typename T>
 inline int pass_first_variant(int N) { return sizeof(T) == 8 && pass_has_wide(N) ? 1 : 0; }
 
@@ -527,6 +531,9 @@ size_t pass_smem(int N, int wide, int lines) {
       if (wide == 1) return pass_smem_bytes<T, NN, 1>(lines);                          \
       if (wide == 2) return pass_smem_bytes<T, NN, 2>(lines);                          \
     }                                                                                  \
+    if constexpr (sizeof(T) == 8 && (NN == 128 || NN == 256)) {                        \
+      if (wide == 1) return pass_smem_bytes<T, NN, 1>(lines);                          \
+    }                                                                                  \
     return pass_smem_bytes<T, NN, 0>(lines);
     CSL_FOR_EACH_N(CASE)
 #undef CASE
@@ -534,47 +541,41 @@ size_t pass_smem(int N, int wide, int lines) {
   return 0;
 }
 
+// the FP64 form's radices (lines of 16384 points have none)
+inline FixRadices fix_radices_of(int N, int wide) {
+  switch (N) {
+#define ONE(NN, V) fix_radices<NN, fix_lanes(NN, V)>()
+#define CASE(NN) \
+  case NN: return ONE(NN, 0);
+#define CASE2(NN, V) \
+  case NN: return wide == V ? ONE(NN, V) : ONE(NN, 0);
+    CASE(16) CASE(32) CASE(64) CASE2(128, 1) CASE2(256, 1) CASE2(512, 2) CASE2(1024, 2) CASE(2048) CASE(4096) CASE(8192)
+#undef CASE
+#undef CASE2
+#undef ONE
+  }
+  return {0, {0, 0, 0, 0}};
+}
+inline int fix_entries_of(int N, int wide) {
+  const FixRadices f = fix_radices_of(N, wide);
+  int n = 0;
+  for (int p = 1, ls = f.r[0]; p < f.np; ++p) n += (ls *= f.r[p]);
+  return n;
+}
+// the FP64 form's variant that has a table of its own beside variant 0's, or -1
+inline int fix_second_table(int N) { return N == 128 || N == 256 ? 1 : N == 512 || N == 1024 ? 2 : -1; }
+
 // entries of the extra twiddle tables of length N, and where a variant's begin
 template <typename T>
 inline int pass_tp_total(int N) {
-  if constexpr (sizeof(T) == 4) {
-    return line_tp_size(N, 0) + line_tp_size(N, 1);
-  } else {
-    switch (N) {
-#define CASE(NN) \
-  case NN: return fix_table_entries<NN, LineDst<double, NN, 0>::TPL>();
-      CASE(4) CASE(8) CASE(16) CASE(32) CASE(64) CASE(128) CASE(256)
-#undef CASE
-      case 512: return fix_table_entries<512, 64>() + fix_table_entries<512, 128>();
-      case 1024: return fix_table_entries<1024, 64>() + fix_table_entries<1024, 128>();
-      case 2048: return fix_table_entries<2048, BigShape<2048>::TPL>();
-      case 4096: return fix_table_entries<4096, BigShape<4096>::TPL>();
-      case 8192: return fix_table_entries<8192, BigShape<8192>::TPL>();
-    }
-    return 0;
-  }
+  if (sizeof(T) == 4) return line_tp_size(N, 0) + line_tp_size(N, 1);
+  const int second = fix_second_table(N);
+  return fix_entries_of(N, 0) + (second > 0 ? fix_entries_of(N, second) : 0);
 }
 template <typename T>
 inline int pass_tp_offset(int N, int wide) {
   if (sizeof(T) == 4) return wide == 1 || wide == 2 ? line_tp_size(N, 0) : 0;
-  // variants 0 and 1 have the same radices
-  return wide == 2 ? (N == 512 ? fix_table_entries<512, 64>() : fix_table_entries<1024, 64>()) : 0;
-}
-// the FP64 form's pass tables of length N, in the order of pass_tp_offset
-// (lines of 16384 points have none)
-inline FixRadices fix_radices_of(int N, int wide) {
-  switch (N) {
-    case 32: return fix_radices<32, LineDst<double, 32, 0>::TPL>();
-    case 64: return fix_radices<64, LineDst<double, 64, 0>::TPL>();
-    case 128: return fix_radices<128, LineDst<double, 128, 0>::TPL>();
-    case 256: return fix_radices<256, LineDst<double, 256, 0>::TPL>();
-    case 512: return wide == 2 ? fix_radices<512, 128>() : fix_radices<512, 64>();
-    case 1024: return wide == 2 ? fix_radices<1024, 128>() : fix_radices<1024, 64>();
-    case 2048: return fix_radices<2048, BigShape<2048>::TPL>();
-    case 4096: return fix_radices<4096, BigShape<4096>::TPL>();
-    case 8192: return fix_radices<8192, BigShape<8192>::TPL>();
-  }
-  return {0, {0, 0, 0, 0}};
+  return wide == fix_second_table(N) ? fix_entries_of(N, 0) : 0;
 }
 
 // lanes per line of a variant
@@ -590,6 +591,9 @@ inline int pass_tpl(int N, int wide) {
     if constexpr (NN >= 512) {                         \
       if (wide == 1) return LineDst<T, NN, 1>::TPL;    \
       if (wide == 2) return LineDst<T, NN, 2>::TPL;    \
+    }                                                  \
+    if constexpr (sizeof(T) == 8 && (NN == 128 || NN == 256)) { \
+      if (wide == 1) return LineDst<T, NN, 1>::TPL;    \
     }                                                  \
     return LineDst<T, NN, 0>::TPL;
     CSL_FOR_EACH_N(CASE)

@@ -38,8 +38,8 @@ constexpr int kMaxDevices = 64;
 constexpr int kTwD = kMaxN;                        // N/2 complex = N doubles
 constexpr int kHsD = kMaxN / 2 + 2;
 // extra twiddles, complex: the larger of the FP32 variant's and of the FP64 form's pass tables (N = 1024)
-constexpr int kTpE = wide_tp_size<1024>() > fix_table_entries<1024, 64>() ? wide_tp_size<1024>()
-                                                                           : fix_table_entries<1024, 64>();
+constexpr int kTpE = wide_tp_size<1024>() > fix_tp_entries<FixShape<1024, 64>>() ? wide_tp_size<1024>()
+                                                                           : fix_tp_entries<FixShape<1024, 64>>();
 constexpr int kTpD = 2 * kTpE + 2;
 constexpr int kAxisD = kTwD + kHsD + kTpD + 2 * kMaxN;
 
@@ -256,9 +256,7 @@ cudaError_t run_static(int dim, const int n[3], double gamma, double alpha, doub
     cnorm *= 2.0 / (double)N;
     const int wide = pass_has_wide(N) ? 1 : 0;
     const FixRadices f = fix_radices_of(N, wide);
-    int ntp = 0;
-    for (int p = 1, ls = f.r[0]; p < f.np; ++p) ntp += (ls *= f.r[p]);
-    k_static_axis_tables<T><<<8, 256, 0, s>>>(P.tables + (long)d * kAxisD, N, f, ntp);
+    k_static_axis_tables<T><<<8, 256, 0, s>>>(P.tables + (long)d * kAxisD, N, f, fix_entries_of(N, wide));
     ax[d] = axis_tables<T>(P.tables + (long)d * kAxisD);
   }
   cudaError_t e = cudaGetLastError();

@@ -86,6 +86,24 @@ def test_tile_widths(csl, lines):
     assert np.linalg.norm(out - r1 - 1j * r2) <= 8 * 512 * 2.0**-53 * np.linalg.norm(r1 + 1j * r2)
 
 
+@pytest.mark.parametrize("N,variant", [(128, 0), (128, 1), (256, 0), (256, 1), (512, 1), (512, 2), (1024, 1), (1024, 2)])
+def test_variants(csl, tmp_path, N, variant):
+    """Every number of lanes per line, chosen through the tuner's cache."""
+    n = N - 1
+    v = W.rhs_normal((n, n), 10)
+    beta = 4.0 * 8.0 * N * N
+    r1, r2 = O.precond_apply(v.real.copy(), v.imag.copy(), 1.0, 0.0, beta)
+    ref = r1 + 1j * r2
+    faces = [dev(f) for f in W.sample_faces(2, (n, n), W.coef_const(1.0))]
+    path = tmp_path / "tune.txt"
+    path.write_text(f"csl-tune-cache 1\n8 0 {N} {n} {n} {variant} 2\n8 2 {N} {n} 1 {variant} 2\n")
+    csl.tune_cache_load(str(path))
+    with csl.Plan(faces, 1j * beta) as p:
+        assert p.config.count("lines=2 ") == 2
+        out = p.precondition(dev(v)).cpu().numpy()
+    assert np.linalg.norm(out - ref) <= 8 * N * 2.0**-53 * np.linalg.norm(ref)
+
+
 @pytest.mark.parametrize("ns", [(15, 63), (127, 31), (511, 63), (1023, 15)])
 @pytest.mark.parametrize("bad", [np.nan, np.inf])
 def test_nonfinite_spreads(csl, ns, bad):
