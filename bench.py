@@ -172,6 +172,9 @@ def kernel_model(name, M, d, prec, N, ff=False):
         return b32, f64t, f32t
     sT = 16 if prec == "fp64" else 8
     dst_flops = 11 + 5 * math.log2(N)  # per complex point per sine transform (pre, FFT, split, scan)
+    # the FP64 form's transforms (lines up to 8192 points) run on the integer pipes; on the FP64 pipe
+    # they leave the two conversions per point
+    fx = 2.0 if N <= 8192 else dst_flops
     f64 = f32 = 0.0
     if name == "k_stencil" and ff:
         b = sT + 16 + 16 + 8 * d
@@ -182,20 +185,20 @@ def kernel_model(name, M, d, prec, N, ff=False):
     elif name.startswith("k_row<LOAD_LANCZOS"):
         b = 16 + 16 + 16 + sT
         if prec == "fp64":
-            f64 = 4 + dst_flops
+            f64 = 4 + fx
         else:
             f32 = 2 * 36 + dst_flops  # the Lanczos step in float pairs
     elif name.startswith("k_row<LOAD_T,STORE_Z_UPDATE"):
         b = sT + sT + 48 + sT + 32
         f64 = 14
         if prec == "fp64":
-            f64 += dst_flops
+            f64 += fx
         else:
             f32 += dst_flops
     elif name.startswith("k_row<LOAD_T,STORE_Z>"):  # inverse x transform only (update split off)
         b = 2 * sT
         if prec == "fp64":
-            f64 += dst_flops
+            f64 += 2 + fx
         else:
             f32 += dst_flops
     elif name == "k_update":  # w_{j+1}, x_j: z_j, w_{j-1}, w_j, x in; w_{j+1}, x out
@@ -208,13 +211,13 @@ def kernel_model(name, M, d, prec, N, ff=False):
         b = 2 * sT + (8 if prec == "fp64" else 0)
         fl = 2 * dst_flops + 7
         if prec == "fp64":
-            f64 += fl
+            f64 += 2 * fx + 6
         else:
             f32 += fl
     else:  # plain strided transform (3D y passes)
         b = 2 * sT
         if prec == "fp64":
-            f64 += dst_flops
+            f64 += fx
         else:
             f32 += dst_flops
     return b * M, f64 * M, f32 * M

@@ -82,8 +82,8 @@ void push_root(std::vector<double>& out, long num, long den) {
 
 // The extra twiddle tables of a transform of length N: first the four-step
 // table of the warp-per-line path (N >= 64: [k1][g] = w_N^{g k1}, k1 < R1,
-// g < R2; line_tp_size(N, false) entries), then, for N = 512 and 1024, the
-// Stockham passes 2 and 3 of the two-warp path ([q][k] = w_{Ls r}^{q k}).
+// g < R2; line_tp_size(N, false) entries), then, for N = 128 to 1024, the
+// Stockham passes 2 and 3 of the wide path ([q][k] = w_{Ls r}^{q k}).
 void make_tp_table(int N, std::vector<double>& out) {
   out.clear();
   int R1 = 0, R2 = 0;
@@ -97,10 +97,15 @@ void make_tp_table(int N, std::vector<double>& out) {
   }
   for (int k1 = 0; k1 < R1; ++k1)
     for (int g = 0; g < R2; ++g) push_root(out, (long)g * k1, N);
-  if (N < 512) return;
-  const int R0 = N == 1024 ? WideShape<1024>::R0 : WideShape<512>::R0;
-  const int W1 = N == 1024 ? WideShape<1024>::R1 : WideShape<512>::R1;
-  const int W2 = N == 1024 ? WideShape<1024>::R2 : WideShape<512>::R2;
+  if (N < 128) return;
+  int R0 = 0, W1 = 0, W2 = 0;
+  switch (N) {
+    case 128: R0 = WideShape<128>::R0; W1 = WideShape<128>::R1; W2 = WideShape<128>::R2; break;
+    case 256: R0 = WideShape<256>::R0; W1 = WideShape<256>::R1; W2 = WideShape<256>::R2; break;
+    case 512: R0 = WideShape<512>::R0; W1 = WideShape<512>::R1; W2 = WideShape<512>::R2; break;
+    case 1024: R0 = WideShape<1024>::R0; W1 = WideShape<1024>::R1; W2 = WideShape<1024>::R2; break;
+    default: return;
+  }
   const int passes[2][2] = {{R0, W1}, {R0 * W1, W2}};  // (Ls, r) of passes 2 and 3
   for (int p = 0; p < 2; ++p) {
     const int Ls = passes[p][0], r = passes[p][1];
@@ -762,7 +767,7 @@ std::mutex g_tune_mu;
 // loader, so a shape read from a file is rebuilt and checked the same way.
 template <typename T>
 bool make_candidate(const PassCfg& c, int kind, int w, int lines, PassCfg& cand) {
-  if (w < 0 || w >= pass_num_variants<T>(c.N) || lines < 1 || (lines & (lines - 1))) return false;
+  if (w < 0 || w >= pass_num_variants(c.N) || lines < 1 || (lines & (lines - 1))) return false;
   const int tpl = pass_tpl<T>(c.N, w);
   if (lines * tpl < 32 || lines * tpl > 256) return false;
   cand = c;
@@ -825,10 +830,14 @@ cudaError_t tune_pass(csl_plan* P, PassCfg& c, int kind, cudaEvent_t* ev, const 
   double best_ms = 1e30;
   double ms[8];
   cudaError_t e = cudaSuccess;
-  for (int w = pass_first_variant<T>(keep.N); w < pass_num_variants<T>(keep.N) && e == cudaSuccess; ++w) {
+  for (int w = pass_first_variant<T>(keep.N); w < pass_num_variants(keep.N) && e == cudaSuccess; ++w) {
     for (int lines = 1; lines <= 256 && e == cudaSuccess; lines <<= 1) {
       PassCfg cand;
       if (!make_candidate<T>(keep, kind, w, lines, cand)) continue;
+      // a batch takes its systems' shapes, so that its results are theirs to
+      // the bit; tiles of less than a 32-byte sector a row, a little faster for
+      // one system of long lines, cost 64 systems twice the time (n = 511: 536 us)
+      if (kind != 0 && sizeof(T) == 4 && keep.N >= 512 && lines < 4 && keep.ncols >= 4) continue;
       c = cand;  // c is the plan's own pass configuration
       double t = 1e30;
       for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {  // the faster of two measurements
@@ -893,7 +902,7 @@ bool tune_entry_valid(const TuneKey& k, int wide, int lines) {
   if (k.kind < 0 || k.kind > 2) return false;
   if (k.N < 4 || k.N > 1024 || ilog2_exact(k.N) < 0) return false;
   if (k.ncols < 1 || k.nouter < 1) return false;
-  if (wide < 0 || wide >= (k.prec == 8 ? pass_num_variants<double>(k.N) : pass_num_variants<float>(k.N))) return false;
+  if (wide < 0 || wide >= pass_num_variants(k.N)) return false;
   return lines >= 1 && lines <= 256 && !(lines & (lines - 1));
 }
 
@@ -1236,7 +1245,7 @@ csl_status csl_plan_create(csl_plan** out, int dim, const int64_t n[3], const do
     }
   }
   {
-    P->sten_strip = strip_rows(dim, nx, ny, nz, kSMs * stencil_warps(dim, P->ff != 0));
+    P->sten_strip = strip_rows(dim, nx, ny, nz, kSMs * stencil_warps(dim, P->ff != 0), P->ff ? 4 : 1);
     P->sten_blocks = stencil_blocks(P, P->sten_strip);
   }
   Grid g;
@@ -1672,7 +1681,6 @@ struct BatchGroup {
   std::vector<int> sys;  // indices of the group's systems
   csl_plan* proto = nullptr;
   int ff = 1;  // all systems of the group take the float-pair stencil
-  int sten_strip = 1, sten_blocks = 1;  // the stencil's strips per system
   UpdateArgs* d_upd[2] = {nullptr, nullptr};
   StencilArgs* d_sten[2] = {nullptr, nullptr};
   void* d_p1[2] = {nullptr, nullptr};   // RowArgs<T>
@@ -1777,11 +1785,6 @@ cudaError_t build_group_args(csl_batch* B, BatchGroup& G) {
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < ns; ++i)
     if (!B->plans[G.sys[i]]->ff) G.ff = 0;
-  {
-    const csl_plan* P = G.proto;
-    G.sten_strip = strip_rows(P->dim, P->n[0], P->n[1], P->n[2], (long)kSMs * stencil_warps(P->dim, G.ff != 0) / ns);
-    G.sten_blocks = stencil_blocks(P, G.sten_strip);
-  }
   for (int par = 0; par < 2 && e == cudaSuccess; ++par) {
     std::vector<StencilArgs> sa(ns);
     std::vector<RowArgs<T>> p1(ns), p3(ns);
@@ -1790,7 +1793,6 @@ cudaError_t build_group_args(csl_batch* B, BatchGroup& G) {
       csl_plan* P = B->plans[G.sys[i]];
       StencilArgs a = stencil_args(P, par);
       a.use_cond = 0;
-      a.strip = G.sten_strip;
       sa[i] = a;
       up[i] = update_args(P, par);
       p1[i] = p1_args<T>(P, par);
@@ -1881,8 +1883,8 @@ cudaError_t group_iteration(csl_batch* B, BatchGroup& G, int par, cudaStream_t s
   memset(&sd, 0, sizeof(sd));
   const StencilArgs* sb = (const StencilArgs*)G.d_sten[par];
   const size_t smem = (sizeof(TZ) == 8 && G.ff) ? ff_stencil_smem(P->dim) : 0;
-  cudaError_t e = launch_k(P->use_pdl != 0, stencil_fn<TZ>(P->dim, G.ff != 0, P->vpair != 0), G.sten_blocks * ns, 256,
-                           smem, s, sd, sb, G.sten_blocks);
+  cudaError_t e = launch_k(P->use_pdl != 0, stencil_fn<TZ>(P->dim, G.ff != 0, P->vpair != 0), P->sten_blocks * ns, 256,
+                           smem, s, sd, sb, P->sten_blocks);
   RowArgs<T> rd;
   memset(&rd, 0, sizeof(rd));
   if (e == cudaSuccess)
@@ -1894,113 +1896,6 @@ cudaError_t group_iteration(csl_batch* B, BatchGroup& G, int par, cudaStream_t s
   // the update moves the same bytes as fused into the inverse x pass, at the
   // rate of a streaming kernel
   if (e == cudaSuccess) e = launch_update<T>(P, par, s, G.d_upd[par], ns);
-  return e;
-}
-
-// The batched passes' shapes are tuned on the group's own launches: with many
-// systems the CTAs are plenty, and what counts is wide tiles and few
-// instructions, not the latency of one line (n = 511, 64 systems: the shape of
-// a single system's MID pass, one column per CTA, takes 536 us there).  Cached
-// per (pass, number of systems) for the life of the process.
-std::map<std::pair<TuneKey, int>, PassCfg> g_batch_tune_cache;
-
-template <typename T>
-cudaError_t tune_group_pass(csl_batch* B, BatchGroup& G, int kind, void* scratch, cudaEvent_t* ev) {
-  csl_plan* proto = G.proto;
-  PassCfg csl_plan::*field = kind == 0 ? &csl_plan::row : kind == 1 || proto->dim == 2 ? &csl_plan::sy : &csl_plan::sz;
-  const PassCfg keep = proto->*field;
-  if (keep.L.tc || keep.wide >= 3) return cudaSuccess;
-  const int ns = (int)G.sys.size();
-  const std::pair<TuneKey, int> key = {{(int)sizeof(T), kind, keep.N, keep.ncols, keep.nouter}, ns};
-  cudaError_t e = cudaSuccess;
-  PassCfg best = keep;
-  bool hit = false;
-  {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_batch_tune_cache.find(key);
-    hit = it != g_batch_tune_cache.end() && make_candidate<T>(keep, kind, it->second.wide, it->second.lines, best);
-  }
-  double best_ms = 1e30;
-  for (int w = pass_first_variant<T>(keep.N); w < pass_num_variants<T>(keep.N) && !hit && e == cudaSuccess; ++w) {
-    for (int lines = 1; lines <= 256 && e == cudaSuccess; lines <<= 1) {
-      PassCfg cand;
-      if (!make_candidate<T>(keep, kind, w, lines, cand)) continue;
-      for (int i : G.sys) B->plans[i]->*field = cand;
-      // arguments of the candidate: the x passes P1 and P3, or the strided pass
-      std::vector<RowArgs<T>> ra;
-      std::vector<StridedArgs<T>> sa;
-      for (int i : G.sys) {
-        csl_plan* P = B->plans[i];
-        if (kind == 0) {
-          ra.push_back(p1_args<T>(P, 0));
-        } else {
-          const int ax = kind == 1 || P->dim == 2 ? 1 : 2;
-          sa.push_back(strided_args<T>(P, cand, ax));
-          if (kind == 2) fill_mid<T>(P, sa.back(), ax);
-          sa.back().st = P->st;
-          sa.back().scalar_mode = kind == 2 ? 3 : 0;
-        }
-      }
-      if (kind == 0)
-        for (int i : G.sys) ra.push_back(p3_args<T>(B->plans[i], 0));
-      const void* src = kind == 0 ? (const void*)ra.data() : (const void*)sa.data();
-      e = cudaMemcpyAsync(scratch, src, kind == 0 ? sizeof(ra[0]) * ra.size() : sizeof(sa[0]) * sa.size(),
-                          cudaMemcpyHostToDevice, B->stream);
-      RowArgs<T> rd;
-      StridedArgs<T> sd;
-      memset(&rd, 0, sizeof(rd));
-      memset(&sd, 0, sizeof(sd));
-      double t = 1e30;
-      for (int rep = 0; rep < 4 && e == cudaSuccess; ++rep) {  // the fastest of three, after one untimed
-        e = cudaEventRecord(ev[0], B->stream);
-        if (kind == 0) {
-          const RowArgs<T>* d = (const RowArgs<T>*)scratch;
-          if (e == cudaSuccess)
-            e = launch_row<T>(cand.N, cand.wide, lanczos_load(proto), STORE_T, rd, cand.L, B->stream, d, ns);
-          if (e == cudaSuccess) e = launch_row<T>(cand.N, cand.wide, LOAD_T, STORE_Z, rd, cand.L, B->stream, d + ns, ns);
-        } else {
-          if (e == cudaSuccess)
-            e = launch_strided<T>(cand.N, cand.wide, kind == 2, sd, cand.L, B->stream, (const StridedArgs<T>*)scratch, ns);
-        }
-        if (e == cudaSuccess) e = cudaEventRecord(ev[1], B->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(B->stream);
-        float ms = 0.f;
-        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
-        if (rep > 0 && ms < t) t = ms;
-      }
-      if (e == cudaSuccess && t < best_ms) {
-        best_ms = t;
-        best = cand;
-      }
-    }
-  }
-  for (int i : G.sys) B->plans[i]->*field = best;
-  if (e == cudaSuccess && !hit) {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_batch_tune_cache[key] = best;
-  }
-  return e;
-}
-
-template <typename T>
-cudaError_t tune_group(csl_batch* B, BatchGroup& G) {
-  const size_t ns = G.sys.size();
-  void* scratch = nullptr;
-  cudaEvent_t ev[2] = {nullptr, nullptr};
-  cudaError_t e = cudaMalloc(&scratch, ns * (2 * sizeof(RowArgs<T>) > sizeof(StridedArgs<T>) ? 2 * sizeof(RowArgs<T>)
-                                                                                              : sizeof(StridedArgs<T>)));
-  for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaEventCreate(&ev[i]);
-  // finite inputs for every pass
-  for (size_t i = 0; i < ns && e == cudaSuccess; ++i) {
-    csl_plan* P = B->plans[G.sys[i]];
-    for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = cudaMemsetAsync(P->v[k], 0, sizeof(double2) * P->M, B->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(P->T, 0, sizeof(typename C2<T>::t) * P->M, B->stream);
-  }
-  for (int kind = 0; kind < 3; ++kind)
-    if (e == cudaSuccess && !(kind == 1 && G.proto->dim == 2)) e = tune_group_pass<T>(B, G, kind, scratch, ev);
-  for (cudaEvent_t x : ev)
-    if (x) cudaEventDestroy(x);
-  if (scratch) cudaFree(scratch);
   return e;
 }
 
@@ -2208,8 +2103,6 @@ csl_status csl_batch_create(csl_batch** out, int nsys, const csl_system_desc* sy
     }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&G.branch, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&G.ev, cudaEventDisableTiming);
-    if (e == cudaSuccess && o.autotune && o.lines_per_cta <= 0 && G.sys.size() > 1)
-      e = fp32 ? tune_group<float>(B, G) : tune_group<double>(B, G);
     if (e == cudaSuccess) e = fp32 ? build_group_args<float>(B, G) : build_group_args<double>(B, G);
   }
   if (e != cudaSuccess) {

@@ -24,14 +24,15 @@
 // the finer scale.  The split and the prefix sum only add, modulo 2^64, and
 // their results fit.
 //
-// Measured on a GB300, FP64 form, per iteration of MINRES: n = 1023 in 2D, x
-// pass with the Lanczos step 124.6 us in FP64 arithmetic, 36.3 here; MID pass
-// 252.5 and 72.2; inverse x pass 119.0 and 35.1; whole iteration 524 and 178.
-// n = 127 in 3D 1067 and 413 us; n = 4095 9297 and 3237.  Error of one line
-// against long double: 0.05 to 0.9 times that of the FP64 butterflies for
-// random, smooth, decaying and constant lines of 4 to 8192 points, about the
-// same for a spike of 4096.  What bounds it now is latency: 11 to 16 warps per
-// SM (registers and shared memory hold the lines), integer pipe 30% busy.
+// Measured on a GB300, FP64 form, per iteration of MINRES, FP64 arithmetic and
+// this (with the lanes of fix_lanes and the tables in the L1): n = 1023 in 2D, x
+// pass with the Lanczos step 124.6 and 33.9 us, MID pass 252.5 and 66.7, inverse
+// x pass 119.0 and 27.2, whole iteration 524 and 166; n = 63, 71 and 35 us;
+// n = 127 in 3D 1067 and 360; n = 4095 9297 and 2553.  Error of one line against
+// long double: 0.05 to 0.9 times that of the FP64 butterflies for random,
+// smooth, decaying and constant lines of 4 to 8192 points, about the same for a
+// spike of 4096.  What bounds it now is latency: 13 to 20 warps per SM
+// (registers and shared memory hold the lines), integer pipe 30% busy.
 //
 // A line with an infinity or NaN returns NaN everywhere (the FP64 butterflies
 // spread it over the line too); a zero line returns zeros.

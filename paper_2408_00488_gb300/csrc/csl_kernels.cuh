@@ -242,16 +242,19 @@ __host__ __device__ inline long stencil_strips(int dim, int nx, int ny, int nz, 
   return nsx * ((nm + strip - 1) / strip) * (dim == 3 ? ny : 1);
 }
 
-// Strip length for `warps` resident warps (stencil_warps per SM; the systems of
-// a batch share them): the fewest steps of the longest-running warp, i.e. the
-// waves of warps times a strip's steps and the two it takes to fill the operand
-// ring.  n = 63: strips of one step, 9.9 us, where strips of four took 13.9.  3D, n = 127, float pairs: strips of 19 planes gave 3556 warps to 2432
-// places, two waves of 21 steps; strips of 32 give one of 34.
-inline int strip_rows(int dim, int nx, int ny, int nz, long warps) {
+// Strip length for `warps` resident warps: the fewest steps of the longest-
+// running warp, i.e. the waves of warps times a strip's steps and the two it
+// takes to fill the operand ring.  At least `least` steps: 1 for the FP64
+// kernels (n = 63: 9.9 us, 13.9 with strips of four), 4 for the float pairs,
+// whose ring is three steps deep and whose strips a batch's systems take over
+// (a batch's sums are those of its systems alone, to the bit).  3D, n = 127,
+// float pairs: strips of 19 planes gave 3556 warps to 2432 places, two waves of
+// 21 steps, 55 us; two waves of 17 take 51.
+inline int strip_rows(int dim, int nx, int ny, int nz, long warps, int least) {
   const long cols = (long)((nx + 31) / 32) * (dim == 3 ? ny : 1);
   const long nm = dim == 2 ? ny : nz;
   long best = nm, cost = -1;
-  for (long strip = 1; strip <= nm; ++strip) {
+  for (long strip = nm < least ? nm : least; strip <= nm; ++strip) {
     const long strips = cols * ((nm + strip - 1) / strip);
     const long c = ((strips + warps - 1) / (warps > 0 ? warps : 1)) * (strip + 2);
     if (cost < 0 || c < cost) {
