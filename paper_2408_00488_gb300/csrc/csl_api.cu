@@ -82,8 +82,8 @@ void push_root(std::vector<double>& out, long num, long den) {
 
 // The extra twiddle tables of a transform of length N: first the four-step
 // table of the warp-per-line path (N >= 64: [k1][g] = w_N^{g k1}, k1 < R1,
-// g < R2; line_tp_size(N, false) entries), then, for N = 128 to 1024, the
-// Stockham passes 2 and 3 of the wide path ([q][k] = w_{Ls r}^{q k}).
+// g < R2; line_tp_size(N, false) entries), then, for N = 512 and 1024, the
+// Stockham passes 2 and 3 of the two-warp path ([q][k] = w_{Ls r}^{q k}).
 void make_tp_table(int N, std::vector<double>& out) {
   out.clear();
   int R1 = 0, R2 = 0;
@@ -97,15 +97,10 @@ void make_tp_table(int N, std::vector<double>& out) {
   }
   for (int k1 = 0; k1 < R1; ++k1)
     for (int g = 0; g < R2; ++g) push_root(out, (long)g * k1, N);
-  if (N < 128) return;
-  int R0 = 0, W1 = 0, W2 = 0;
-  switch (N) {
-    case 128: R0 = WideShape<128>::R0; W1 = WideShape<128>::R1; W2 = WideShape<128>::R2; break;
-    case 256: R0 = WideShape<256>::R0; W1 = WideShape<256>::R1; W2 = WideShape<256>::R2; break;
-    case 512: R0 = WideShape<512>::R0; W1 = WideShape<512>::R1; W2 = WideShape<512>::R2; break;
-    case 1024: R0 = WideShape<1024>::R0; W1 = WideShape<1024>::R1; W2 = WideShape<1024>::R2; break;
-    default: return;
-  }
+  if (N < 512) return;
+  const int R0 = N == 1024 ? WideShape<1024>::R0 : WideShape<512>::R0;
+  const int W1 = N == 1024 ? WideShape<1024>::R1 : WideShape<512>::R1;
+  const int W2 = N == 1024 ? WideShape<1024>::R2 : WideShape<512>::R2;
   const int passes[2][2] = {{R0, W1}, {R0 * W1, W2}};  // (Ls, r) of passes 2 and 3
   for (int p = 0; p < 2; ++p) {
     const int Ls = passes[p][0], r = passes[p][1];
@@ -767,7 +762,7 @@ std::mutex g_tune_mu;
 // loader, so a shape read from a file is rebuilt and checked the same way.
 template <typename T>
 bool make_candidate(const PassCfg& c, int kind, int w, int lines, PassCfg& cand) {
-  if (w < 0 || w >= pass_num_variants(c.N) || lines < 1 || (lines & (lines - 1))) return false;
+  if (w < 0 || w >= pass_num_variants<T>(c.N) || lines < 1 || (lines & (lines - 1))) return false;
   const int tpl = pass_tpl<T>(c.N, w);
   if (lines * tpl < 32 || lines * tpl > 256) return false;
   cand = c;
@@ -830,7 +825,7 @@ cudaError_t tune_pass(csl_plan* P, PassCfg& c, int kind, cudaEvent_t* ev, const 
   double best_ms = 1e30;
   double ms[8];
   cudaError_t e = cudaSuccess;
-  for (int w = pass_first_variant<T>(keep.N); w < pass_num_variants(keep.N) && e == cudaSuccess; ++w) {
+  for (int w = pass_first_variant<T>(keep.N); w < pass_num_variants<T>(keep.N) && e == cudaSuccess; ++w) {
     for (int lines = 1; lines <= 256 && e == cudaSuccess; lines <<= 1) {
       PassCfg cand;
       if (!make_candidate<T>(keep, kind, w, lines, cand)) continue;
@@ -902,7 +897,7 @@ bool tune_entry_valid(const TuneKey& k, int wide, int lines) {
   if (k.kind < 0 || k.kind > 2) return false;
   if (k.N < 4 || k.N > 1024 || ilog2_exact(k.N) < 0) return false;
   if (k.ncols < 1 || k.nouter < 1) return false;
-  if (wide < 0 || wide >= pass_num_variants(k.N)) return false;
+  if (wide < 0 || wide >= (k.prec == 8 ? pass_num_variants<double>(k.N) : pass_num_variants<float>(k.N))) return false;
   return lines >= 1 && lines <= 256 && !(lines & (lines - 1));
 }
 

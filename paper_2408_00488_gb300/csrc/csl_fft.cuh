@@ -260,7 +260,7 @@ __device__ __forceinline__ void dst_line(typename C2<T>::t* a, int t, const type
 }
 
 // ---------------------------------------------------------------------------
-// Wide paths (N = 128 .. 1024): TPL = 32, 64 or 128 lanes (one to four warps) per
+// Wide paths (N = 512, 1024): TPL = 64 or 128 lanes (two or four warps) per
 // line, a three-pass Stockham autosort FFT with radices R0 x R1 x R2,
 // CTA-wide barriers.  On a 2D grid there are only n lines per pass, so one
 // warp per line leaves most of the GPU idle; more lanes per line cut the
@@ -272,14 +272,11 @@ __device__ __forceinline__ void dst_line(typename C2<T>::t* a, int t, const type
 // (wpad) so the strided stores of the early passes spread over the banks.
 // ---------------------------------------------------------------------------
 template <int N> struct WideShape;
-template <> struct WideShape<128> { enum { R0 = 8, R1 = 4, R2 = 4 }; };
-template <> struct WideShape<256> { enum { R0 = 8, R1 = 8, R2 = 4 }; };
 template <> struct WideShape<512> { enum { R0 = 8, R1 = 8, R2 = 8 }; };
 template <> struct WideShape<1024> { enum { R0 = 8, R1 = 8, R2 = 16 }; };
 
-// lanes per line of wide variant v (1: two warps, 2: four warps; one warp for
-// lines of 128 and 256 points, where the four-step path has 8 and 16 lanes)
-__host__ __device__ constexpr int wide_tpl(int N, int v) { return N < 512 ? 32 : v == 2 ? 128 : 64; }
+// lanes per line of wide variant v (1: two warps, 2: four warps)
+__host__ __device__ constexpr int wide_tpl(int v) { return v == 2 ? 128 : 64; }
 
 __host__ __device__ constexpr int wpad(int i) { return i + (i >> 5); }
 
@@ -475,7 +472,7 @@ template <typename T, int N, int V>
 struct LineDst {
   typedef typename C2<T>::t c_t;
   typedef SmemTables<T, N, wide_tp_size<N>()> Tables;
-  enum { TPL = wide_tpl(N, V), LS = wide_line_stride<N, wide_tpl(N, V)>(), SCRATCH = 4 };
+  enum { TPL = wide_tpl(V), LS = wide_line_stride<N, wide_tpl(V)>(), SCRATCH = 4 };
   static __device__ __forceinline__ int in_pos(int j) { return wpad(j); }
   static __device__ __forceinline__ int out_pos(int m) { return wide_out_pos<N, TPL>(m); }
   template <bool PERM_IN>
@@ -669,9 +666,7 @@ struct LineDst<double, N, 3> : FixDst<N, fix_lanes(N, 3)> {};
 
 // Host-side size of the extra twiddle table of length N in the FP32 forms.
 __host__ __device__ constexpr int line_tp_size(int N, int wide) {
-  if (!wide) return N >= 64 ? N : 0;
-  return N >= 1024 ? wide_tp_size<1024>() : N >= 512 ? wide_tp_size<512>() : N >= 256 ? wide_tp_size<256>()
-         : N >= 128 ? wide_tp_size<128>() : 0;
+  return wide ? (N >= 1024 ? wide_tp_size<1024>() : N >= 512 ? wide_tp_size<512>() : 0) : (N >= 64 ? N : 0);
 }
 
 }  // namespace csl

@@ -5,8 +5,6 @@ namespace csl {
 #define CASE(NN) CSL_INSTANTIATE_PASS(float, NN, 0)
 CSL_FOR_EACH_N(CASE)
 #undef CASE
-CSL_INSTANTIATE_PASS(float, 128, 1)
-CSL_INSTANTIATE_PASS(float, 256, 1)
 CSL_INSTANTIATE_PASS(float, 512, 1)
 CSL_INSTANTIATE_PASS(float, 512, 2)
 CSL_INSTANTIATE_PASS(float, 1024, 1)

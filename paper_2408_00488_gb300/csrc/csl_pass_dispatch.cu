@@ -19,7 +19,7 @@ cudaError_t launch_row(int N, int wide, int load, int store, const RowArgs<T>& a
       if (wide == 1) return launch_row_n<T, NN, 1>(load, store, a, L, s, batch, nsys); \
       if (wide == 2) return launch_row_n<T, NN, 2>(load, store, a, L, s, batch, nsys); \
     }                                                                                  \
-    if constexpr (NN == 128 || NN == 256) {                        \
+    if constexpr (sizeof(T) == 8 && (NN == 128 || NN == 256)) {                        \
       if (wide == 1) return launch_row_n<T, NN, 1>(load, store, a, L, s, batch, nsys); \
     }                                                                                  \
     return launch_row_n<T, NN, variant_of<T, NN, 0>>(load, store, a, L, s, batch, nsys);
@@ -43,7 +43,7 @@ cudaError_t launch_strided(int N, int wide, bool mid, const StridedArgs<T>& a, c
       if (wide == 1) return launch_strided_n<T, NN, 1>(mid, a, L, s, batch, nsys);  \
       if (wide == 2) return launch_strided_n<T, NN, 2>(mid, a, L, s, batch, nsys);  \
     }                                                                               \
-    if constexpr (NN == 128 || NN == 256) {                     \
+    if constexpr (sizeof(T) == 8 && (NN == 128 || NN == 256)) {                     \
       if (wide == 1) return launch_strided_n<T, NN, 1>(mid, a, L, s, batch, nsys);  \
     }                                                                               \
     return launch_strided_n<T, NN, variant_of<T, NN, 0>>(mid, a, L, s, batch, nsys);
@@ -64,8 +64,10 @@ cudaError_t set_pass_attrs() {
   if (e == cudaSuccess) e = set_pass_attrs_n<T, 512, 2>();
   if (e == cudaSuccess) e = set_pass_attrs_n<T, 1024, 1>();
   if (e == cudaSuccess) e = set_pass_attrs_n<T, 1024, 2>();
-  if (e == cudaSuccess) e = set_pass_attrs_n<T, 128, 1>();
-  if (e == cudaSuccess) e = set_pass_attrs_n<T, 256, 1>();
+  if constexpr (sizeof(T) == 8) {
+    if (e == cudaSuccess) e = set_pass_attrs_n<T, 128, 1>();
+    if (e == cudaSuccess) e = set_pass_attrs_n<T, 256, 1>();
+  }
   if (e == cudaSuccess) e = set_pass_attrs_big<T>();
   return e;
 }

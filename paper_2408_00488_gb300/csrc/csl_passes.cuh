@@ -502,11 +502,12 @@ struct PassLaunch {
 #define CSL_FOR_EACH_N(X) X(4) X(8) X(16) X(32) X(64) X(128) X(256) X(512) X(1024)
 
 // N = 512 and 1024 exist in three variants (warp per line, 64 and 128 lanes
-// per line: wide = 0, 1, 2; in FP64 0 stands for 1), N = 128 and 256 in two
-// (8 or 16 and 32 lanes; fix_lanes in FP64); the autotuner picks one per pass.
+// per line: wide = 0, 1, 2; in FP64 0 stands for 1), N = 128 and 256 in two in
+// FP64 (fix_lanes); the autotuner picks one per pass.
 inline bool pass_has_wide(int N) { return N == 512 || N == 1024; }
+template <typename T>
 inline int pass_num_variants(int N) {
-  return pass_has_wide(N) ? 3 : N == 128 || N == 256 ? 2 : 1;
+  return pass_has_wide(N) ? 3 : sizeof(T) == 8 && (N == 128 || N == 256) ? 2 : 1;
 }
 // the first variant the tuner tries
 template <typename T>
@@ -530,7 +531,7 @@ size_t pass_smem(int N, int wide, int lines) {
       if (wide == 1) return pass_smem_bytes<T, NN, 1>(lines);                          \
       if (wide == 2) return pass_smem_bytes<T, NN, 2>(lines);                          \
     }                                                                                  \
-    if constexpr (NN == 128 || NN == 256) {                        \
+    if constexpr (sizeof(T) == 8 && (NN == 128 || NN == 256)) {                        \
       if (wide == 1) return pass_smem_bytes<T, NN, 1>(lines);                          \
     }                                                                                  \
     return pass_smem_bytes<T, NN, 0>(lines);
@@ -591,7 +592,7 @@ inline int pass_tpl(int N, int wide) {
       if (wide == 1) return LineDst<T, NN, 1>::TPL;    \
       if (wide == 2) return LineDst<T, NN, 2>::TPL;    \
     }                                                  \
-    if constexpr (NN == 128 || NN == 256) { \
+    if constexpr (sizeof(T) == 8 && (NN == 128 || NN == 256)) { \
       if (wide == 1) return LineDst<T, NN, 1>::TPL;    \
     }                                                  \
     return LineDst<T, NN, 0>::TPL;
