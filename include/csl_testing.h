@@ -53,6 +53,21 @@ csl_status csl_test_convert_f2d(const float* in, double* out, int64_t n, void* s
  */
 csl_status csl_probe_sync_cost(int kernels, int barriers, int unreachable, double out[3]);
 
+/*
+ * Time-out hooks: how a solve ends when a bounded device wait gave up.  No wait
+ * is made; the time-out is recorded as such a wait records it.  out (HOST) =
+ * {done, status} of the solver state afterwards.
+ * csl_test_timeout_raised: `blocks` (1 .. 1024) CTAs copy the state and run the
+ *   scalar step of an iteration; CTA `late` records the time-out in between
+ *   (late < 0: none does).
+ * csl_test_timeout_seen: kernel `kernel` (order of csl_time_kernels) of the
+ *   plan's iteration on a scratch state in which an earlier kernel recorded one.
+ *   It changes the plan's work vectors, not its results.
+ * Synchronous.  Return CSL_OK, CSL_INVALID_ARG or CSL_CUDA_ERROR.
+ */
+csl_status csl_test_timeout_raised(int blocks, int late, int out[2]);
+csl_status csl_test_timeout_seen(csl_plan* plan, int kernel, int out[2]);
+
 #ifdef __cplusplus
 }
 #endif

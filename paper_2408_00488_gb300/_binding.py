@@ -69,6 +69,8 @@ _SIGS = {
     "csl_test_convert_d2f": (ctypes.c_int, [_P, _P, ctypes.c_int64, _P]),
     "csl_test_convert_f2d": (ctypes.c_int, [_P, _P, ctypes.c_int64, _P]),
     "csl_probe_sync_cost": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_double)]),
+    "csl_test_timeout_raised": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_int)]),
+    "csl_test_timeout_seen": (ctypes.c_int, [_P, ctypes.c_int, ctypes.POINTER(ctypes.c_int)]),
     "csl_version": (ctypes.c_char_p, []),
     "csl_status_string": (ctypes.c_char_p, [ctypes.c_int]),
     "csl_last_error": (ctypes.c_char_p, []),

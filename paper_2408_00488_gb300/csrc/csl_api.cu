@@ -1648,12 +1648,33 @@ csl_status csl_time_kernels(csl_plan* P, int reps, double ms[8], const char* nam
     (void)cudaGetLastError();
     return CSL_CUDA_ERROR;
   }
-  if (after.done) {
+  if (after.done || after.timeout) {
     csl_internal_set_error("csl_time_kernels: the scratch iteration ended early; the timings are not valid");
     return CSL_BREAKDOWN;
   }
   for (int k = 0; k < nk; ++k) names[k] = (P->split_update && k == nkb - 1) ? p3split : P->dim == 2 ? n2[k] : n3[k];
   *count = nk;
+  return CSL_OK;
+}
+
+csl_status csl_test_timeout_seen(csl_plan* P, int kernel, int out[2]) {
+  if (!P || !out || kernel < 0 || kernel >= iteration_kernels(P)) return CSL_INVALID_ARG;
+  DevState h = scratch_state(P);
+  h.timeout = 1;
+  DevState* keep = P->st;
+  P->st = P->st_prof;
+  cudaError_t err = cudaMemcpyAsync(P->st, &h, sizeof(h), cudaMemcpyHostToDevice, P->stream);
+  if (err == cudaSuccess) err = launch_iteration_kernel(P, kernel, 0, 2);
+  if (err == cudaSuccess) err = cudaMemcpyAsync(&h, P->st, sizeof(h), cudaMemcpyDeviceToHost, P->stream);
+  if (err == cudaSuccess) err = cudaStreamSynchronize(P->stream);
+  P->st = keep;
+  if (err != cudaSuccess) {
+    record_error(err, "csl_test_timeout_seen", __LINE__);
+    (void)cudaGetLastError();
+    return CSL_CUDA_ERROR;
+  }
+  out[0] = h.done;
+  out[1] = h.status;
   return CSL_OK;
 }
 

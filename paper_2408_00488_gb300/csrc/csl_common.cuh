@@ -108,6 +108,7 @@ struct alignas(16) DevState {
   int entries;    // Givens steps started (MID passes): a loop bound that needs no reduction
   int iter;       // completed iterations = index of the current iterate x
   int maxit, done, status, check, lucky, checks, calibrated, loops;
+  int timeout;    // set by a CTA whose bounded wait gave up (record_timeout)
   unsigned int tickets[4];
 };
 
@@ -135,7 +136,8 @@ __device__ __forceinline__ void cp_async_wait() {
 // not wait on a global round trip.  Only that step changes the scalars while
 // the kernel runs; the reduction tickets do change (other CTAs may have
 // arrived before this one started), so a scalar step writes back the fields
-// it sets, never the whole copy.  Block-wide and asynchronous: it joins the
+// it sets, never the whole copy, and reads a time-out that its own kernel may
+// have recorded from memory.  Block-wide and asynchronous: it joins the
 // next cp.async group, and a wait for that group and a barrier must separate
 // it from the reads.  (Through registers, the warps' later loads would wait
 // for it.)
@@ -143,6 +145,13 @@ __device__ __forceinline__ void state_prefetch(DevState* dst, const DevState* st
   constexpr int W = (int)(sizeof(DevState) / 16);
   for (int i = threadIdx.x; i < W; i += blockDim.x) cp_async16((uint4*)dst + i, (const uint4*)st + i, true);
 }
+
+// A bounded wait gave up: the scalar step of this kernel or of the next one that
+// has a scalar step ends the solve with ST_TIMEOUT.  The kernel itself leaves
+// `done` alone: CTAs of one launch that read different values of it would leave
+// the reduction's ticket unarmed, and the scalar step would store its copy of
+// `done` over it.
+__device__ __forceinline__ void record_timeout(DevState* st) { st->timeout = 1; }
 
 enum { TICKET_STENCIL = 0, TICKET_MID = 1, TICKET_INGEST = 2, TICKET_AUX = 3 };  // TICKET_AUX: warm start
 

@@ -725,9 +725,9 @@ __global__ void __launch_bounds__(256, FF ? (DIM == 2 ? 3 : 2) : 2)
       q.calibrated = 1;
     }
   }
-  if (!q.done && !(q.delta == q.delta)) {
+  if (!q.done && (q.timeout || !(q.delta == q.delta))) {
     q.done = 1;
-    q.status = ST_BREAKDOWN;
+    q.status = q.timeout ? ST_TIMEOUT : ST_BREAKDOWN;
   }
   q.loops += 1;
   if (q.iter > q.maxit + 1 || q.loops > q.maxit + 4) q.done = 1;  // hard caps (integers only)
@@ -1049,6 +1049,7 @@ static __global__ void __launch_bounds__(256) k_ingest(IngestArgs a0, const Inge
   st->rho = 0.0;
   st->iter = 0;
   st->entries = 0;
+  st->timeout = 0;
   st->check = 0;
   st->lucky = 0;
   st->checks = 0;

@@ -24,9 +24,11 @@
 // bounded-wait path, exercised without any fault.
 #include <cuda_runtime.h>
 #include <stdio.h>
+#include <string.h>
 
 #include "../../include/csl_testing.h"
 #include "csl_common.cuh"
+#include "csl_passes.cuh"
 
 void csl_internal_set_error(const char* msg);  // csl_api.cu
 
@@ -67,6 +69,18 @@ __global__ void __launch_bounds__(kProbeThreads) k_probe_barriers(unsigned* coun
     __syncthreads();
     if (give_up) return;
   }
+}
+
+// The end of a tensor-core MID pass of which CTA `late` records a time-out
+// after every CTA has copied the state (late < 0: none does).  No wait is made.
+__global__ void __launch_bounds__(128) k_probe_timeout(csl::StridedArgs<float> a, int late) {
+  __shared__ csl::DevState s_pre;
+  csl::state_prefetch(&s_pre, a.st);
+  csl::cp_async_commit();
+  csl::cp_async_wait<0>();
+  __syncthreads();
+  if ((int)blockIdx.x == late && threadIdx.x == 0) csl::record_timeout(a.st);
+  csl::mid_scalar_tail<float>(a, 1.0 / (128.0 * gridDim.x), (int)blockIdx.x, (int)gridDim.x, &s_pre);
 }
 
 struct ProbeRes {
@@ -184,5 +198,33 @@ extern "C" csl_status csl_probe_sync_cost(int kernels, int barriers, int unreach
     csl_internal_set_error("csl_probe_sync_cost: a grid-barrier wait ran out of its budget");
     return CSL_TIMEOUT;
   }
+  return CSL_OK;
+}
+
+extern "C" csl_status csl_test_timeout_raised(int blocks, int late, int out[2]) {
+  if (!out || blocks < 1 || blocks > 1024 || late >= blocks) return CSL_INVALID_ARG;
+  ProbeRes R;
+  csl::DevState h;
+  memset(&h, 0, sizeof(h));
+  h.gam = h.gam_old = h.gam1 = h.inv_gam = h.lanc = 1.0;
+  h.a1inv_old = h.a1inv_old2 = h.c = h.c_old = h.eta = h.bnorm = 1.0;
+  h.delta = 1.0;
+  h.tol = 1e-300;
+  h.maxit = 1 << 30;
+  const size_t at = (sizeof(h) + 255) / 256 * 256;  // the partials' place
+  PROBE_TRY(cudaStreamCreateWithFlags(&R.s, cudaStreamNonBlocking));
+  PROBE_TRY(cudaMalloc((void**)&R.dbuf, at + (size_t)blocks * sizeof(double)));
+  csl::StridedArgs<float> a;
+  memset(&a, 0, sizeof(a));
+  a.st = (csl::DevState*)R.dbuf;
+  a.partials = (double*)((char*)R.dbuf + at);
+  a.scalar_mode = 2;
+  PROBE_TRY(cudaMemcpyAsync(a.st, &h, sizeof(h), cudaMemcpyHostToDevice, R.s));
+  k_probe_timeout<<<blocks, 128, 0, R.s>>>(a, late);
+  PROBE_TRY(cudaGetLastError());
+  PROBE_TRY(cudaMemcpyAsync(&h, a.st, sizeof(h), cudaMemcpyDeviceToHost, R.s));
+  PROBE_TRY(cudaStreamSynchronize(R.s));
+  out[0] = h.done;
+  out[1] = h.status;
   return CSL_OK;
 }
