@@ -65,7 +65,8 @@ typedef enum csl_status {
 
 typedef enum csl_precision {
   CSL_PREC_FP64 = 0,  /* every step in FP64 (the plain method); the sine transforms of lines up
-                         to 8192 points in 64-bit block fixed point, whose error is no larger */
+                         to 8192 points in 64-bit block fixed point, whose root mean square
+                         error over lines of a kind is below that of FP64 butterflies */
   CSL_PREC_FP32 = 1,  /* sine transforms and per-mode scale of P^{-1} in FP32; the
                          per-point vector work (stencil, Lanczos step, w/x update) in
                          float-pair arithmetic (about 2^-47 relative); Lanczos and Givens

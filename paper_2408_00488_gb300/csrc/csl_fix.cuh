@@ -5,34 +5,45 @@
 // 32 x 32 -> 64 bit products at 60, so an FFT in FP64 arithmetic is bound by
 // that one pipe.  Here the line is scaled by one power of two, held as 64-bit
 // integers, and transformed with integer butterflies.  Sums are exact; a
-// product is rounded once.  Relative to the line's norm the error is below
-// that of the FP64 butterflies, whose every operation rounds to 53 bits.
+// product is rounded once.
 //
 // The algorithm is that of csl_fft.cuh (one length-N complex FFT per line,
 // y_j = h_j (z_j + z_{N-j}) + (z_j - z_{N-j})/4, the C / S split and the
 // prefix sum), as a Stockham FFT with radices R0 .. R3.
 //
-// Scales.  E = largest exponent of the line, so |re|, |im| < 2^(E-1022).
-//   pass 1         values times 2^(S1 - (E-1022)), S1 chosen so that R0 sqrt(2) 2^S1 < 2^62
-//   later passes   shifted right by sh_p while the twiddle is applied, only as
-//                  far as needed: every value of pass p is bounded by both
-//                  sqrt(2) max|z| R0..Rp and by the line's sum of |re| + |im|
-//                  (the bound of every partial DFT sum, and of the result:
-//                  sum_j |y_j| <= sum_j |z_j| because max(s_j, 1/2) <= 1)
-// so nothing overflows for any input, a line of one spike keeps S1 bits, and
-// the rounding of the early passes, which later passes amplify, happens at
-// the finer scale.  The split and the prefix sum only add, modulo 2^64, and
-// their results fit.
+// Scales.  E = largest exponent of the line, so |re|, |im| < 2^(E-1022).  A
+// value is held in units of 2^(E-1022-S1+t); t = 0 at the start and grows by
+// the shifts to the right.  The magnitude of a complex value stays below
+// 2^62.5, so nothing overflows for any input.  The rounding of the early passes
+// is amplified by the later ones, and the prefix sum adds up the errors of N/2
+// modes, so a coarse unit there shows where the line's norm is little more than
+// its largest entry (a point source over a small background).
+//   N <= 1024  S1 is the finest unit at which pass 1 cannot overflow; the later
+//     passes shift while the twiddle is applied, only as far as needed: every
+//     value of pass p is bounded by both sqrt(2) max|z| R0..Rp and by the line's
+//     sum of |re| + |im| (the bound of every partial DFT sum, and of the result:
+//     sum_j |y_j| <= sum_j |z_j| because max(s_j, 1/2) <= 1).
+//   N >= 2048, staged (FixStaged)  these bounds are too coarse: with S1 of pass 1
+//     a spike over a background of 10^-3 at N = 4096 had 14 times the error of
+//     FP64 butterflies.  Here every pass starts with the line's largest value, as
+//     measured after the pass before, just below 2^60, which leaves headroom for
+//     two radix-2 stages, and a radix of 8 or 16 drops one or two bits after the
+//     second one, unless the line's sum bounds the rest.
+// The split and the prefix sum only add, modulo 2^64, and their results fit.
 //
 // Measured on a GB300, FP64 form, per iteration of MINRES, FP64 arithmetic and
 // this (with the lanes of fix_lanes and the tables in the L1): n = 1023 in 2D, x
 // pass with the Lanczos step 124.6 and 33.9 us, MID pass 252.5 and 66.7, inverse
 // x pass 119.0 and 27.2, whole iteration 524 and 166; n = 63, 71 and 35 us;
-// n = 127 in 3D 1067 and 360; n = 4095 9297 and 2553.  Error of one line against
-// long double: 0.05 to 0.9 times that of the FP64 butterflies for random,
-// smooth, decaying and constant lines of 4 to 8192 points, about the same for a
-// spike of 4096.  What bounds it now is latency: 13 to 20 warps per SM
-// (registers and shared memory hold the lines), integer pipe 30% busy.
+// n = 127 in 3D 1067 and 360; n = 4095 9297 and 2553.  Error of one
+// line against 64-bit mantissas or more, over that of FP64 butterflies with the
+// same split and scan, root mean square over 96 lines of a kind (random, constant,
+// alternating, one to eight spikes anywhere or at N/2 and N/4 over random and
+// constant backgrounds of 10^-8 to 0.1, the modes of such lines;
+// tests/fixed_point_host.cu): at most 0.2 for N <= 256, 0.3 at 512, 0.5 at 1024, 0.4
+// at 2048, 0.7 at 4096 and 8192; random and constant lines 0.1 to 0.2.  A single
+// line can come out either way.  What bounds the time is latency: 13 to 20 warps
+// per SM (registers and shared memory hold the lines).
 //
 // A line with an infinity or NaN returns NaN everywhere (the FP64 butterflies
 // spread it over the line too); a zero line returns zeros.
@@ -50,6 +61,7 @@ typedef int4 fxw;       // twiddle: signed 32-bit digits re_hi, re_lo, im_hi, im
 // kFxTw + sh <= 64 bits, i.e. one 32-bit funnel shift by kFxTw - 32 + sh <= 32
 constexpr int kFxTw = 61;
 constexpr int kFxMaxShift = 3;
+constexpr int kFxMaxLeft = 20;
 
 // ---- constants -----------------------------------------------------------------
 __host__ __device__ constexpr unsigned long long fx_mulhi(unsigned long long a, unsigned long long b) {
@@ -157,21 +169,30 @@ __host__ __device__ __forceinline__ long long fx_take(long long acc, long long m
 #endif
 }
 
-// v * w for real v and a constant of F fractional bits (digits h, l), rounded.
-// The product of the two low digits (at most 2^(62-F) units) is left out.
+// v * w for real v and a constant of F fractional bits (digits h, l), rounded
 template <int F>
 __host__ __device__ __forceinline__ long long fx_rmul(long long v, int h, int l) {
   const int vh = fx_hi(v), vl = fx_lo(v);
-  const long long mid = (1ll << (F - 33)) + fx_wide(vh, l) + fx_wide(vl, h);
+  const long long mid = (1ll << (F - 33)) + (fx_wide(vl, l) >> 32) + fx_wide(vh, l) + fx_wide(vl, h);
   return fx_take(fx_wide(vh, h) + (mid >> 32), mid, F - 32);
 }
 
-// w * v / 2^(32 + s), rounded; rnd = 2^(s-1)
+// w * v / 2^(32 + s), rounded; rnd = 2^(s-1).  LOW: with the products of the low
+// digits, up to 2^(31-s) units.  The tables' twiddles change from lane to lane and
+// go without; the constants inside a radix 16 would repeat the same error over all
+// of a pass, which the prefix sum adds up (the modes of a spike at N/2, N = 8192:
+// 1.5 times the error of FP64 butterflies without, 0.5 with).
+template <bool LOW = false>
 __host__ __device__ __forceinline__ fx2 fx_cmul(const fxw& w, fx2 v, unsigned s, long long rnd) {
   const int xh = fx_hi(v.x), xl = fx_lo(v.x), yh = fx_hi(v.y), yl = fx_lo(v.y);
   const int nh = -w.z, nl = -w.w;
-  const long long mr = rnd + fx_wide(xh, w.y) + fx_wide(xl, w.x) + fx_wide(yh, nl) + fx_wide(yl, nh);
-  const long long mi = rnd + fx_wide(xh, w.w) + fx_wide(xl, w.z) + fx_wide(yh, w.y) + fx_wide(yl, w.x);
+  long long mr = rnd, mi = rnd;
+  if constexpr (LOW) {
+    mr += (fx_wide(xl, w.y) + fx_wide(yl, nl)) >> 32;
+    mi += (fx_wide(xl, w.w) + fx_wide(yl, w.y)) >> 32;
+  }
+  mr += fx_wide(xh, w.y) + fx_wide(xl, w.x) + fx_wide(yh, nl) + fx_wide(yl, nh);
+  mi += fx_wide(xh, w.w) + fx_wide(xl, w.z) + fx_wide(yh, w.y) + fx_wide(yl, w.x);
   fx2 r;
   r.x = fx_take((mr >> 32) + fx_wide(xh, w.x) + fx_wide(yh, nh), mr, s);
   r.y = fx_take((mi >> 32) + fx_wide(xh, w.z) + fx_wide(yh, w.x), mi, s);
@@ -183,6 +204,11 @@ __host__ __device__ __forceinline__ fx2 fx_cmul(const fxw& w, fx2 v, unsigned s,
 __host__ __device__ __forceinline__ long long fx_shift(long long v, unsigned sh) {
   const long long half = (1ll << sh) >> 1;
   return (v + (sh ? half - 1 + ((v >> sh) & 1) : 0)) >> sh;
+}
+
+// v / 2^sh for either sign of sh; a shift to the left must fit
+__host__ __device__ __forceinline__ long long fx_rescale(long long v, int sh) {
+  return sh >= 0 ? fx_shift(v, (unsigned)sh) : (long long)((unsigned long long)v << -sh);
 }
 
 __host__ __device__ __forceinline__ fx2 fx_add(fx2 a, fx2 b) {
@@ -225,14 +251,25 @@ __host__ __device__ __forceinline__ fx2 fx_rotate(fx2 v) {
     w.y = c.l;
     w.z = s.h;
     w.w = s.l;
-    r = fx_cmul(w, v, 30, 1ll << 29);
+    r = fx_cmul<true>(w, v, 30, 1ll << 29);
   }
   return r;
 }
 
-template <int S, int K, int R>
-struct FxStage {  // butterflies of the radix-2 stage with half-length S, index K
-  static __host__ __device__ __forceinline__ void run(fx2 (&x)[R]) {
+// Butterflies of the radix-2 stage with half-length S, index K.  HEAD: there is
+// headroom for two stages; before the third, `drop` bits of every value go.
+template <int S, int K, int R, bool HEAD>
+struct FxStage {
+  static __host__ __device__ __forceinline__ void run(fx2 (&x)[R], unsigned drop) {
+    if constexpr (HEAD && S == 4 && K == 0) {
+      if (drop) {
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          x[i].x = fx_shift(x[i].x, drop);
+          x[i].y = fx_shift(x[i].y, drop);
+        }
+      }
+    }
 #pragma unroll
     for (int b = 0; b < R; b += 2 * S) {
       const fx2 u = x[b + K], t = fx_rotate<K, 2 * S>(x[b + K + S]);
@@ -240,15 +277,15 @@ struct FxStage {  // butterflies of the radix-2 stage with half-length S, index 
       x[b + K + S] = fx_sub(u, t);
     }
     if constexpr (K + 1 < S)
-      FxStage<S, K + 1, R>::run(x);
+      FxStage<S, K + 1, R, HEAD>::run(x, drop);
     else if constexpr (2 * S < R)
-      FxStage<2 * S, 0, R>::run(x);
+      FxStage<2 * S, 0, R, HEAD>::run(x, drop);
   }
 };
 
 // in-register forward DFT of length R, natural order in and out
-template <int R>
-__host__ __device__ __forceinline__ void fx_dft(fx2 (&x)[R]) {
+template <int R, bool HEAD = false>
+__host__ __device__ __forceinline__ void fx_dft(fx2 (&x)[R], unsigned drop = 0) {
 #pragma unroll
   for (int i = 0; i < R; ++i) {
     int j = 0;
@@ -260,7 +297,7 @@ __host__ __device__ __forceinline__ void fx_dft(fx2 (&x)[R]) {
       x[j] = t;
     }
   }
-  FxStage<1, 0, R>::run(x);
+  FxStage<1, 0, R, HEAD>::run(x, drop);
 }
 
 // ---- conversions -----------------------------------------------------------------
@@ -320,9 +357,10 @@ __device__ __forceinline__ double fx_to_double(long long v, int q) {
 // two variants: with many lines, as in 3D, fewer lanes and passes win (n = 127
 // in 3D 357 us with 16 lanes, 370 with 32, 384 with 8).  N = 512 and 1024: 64
 // lanes (variant 1, and 0, which has no kernels of its own) or 128 (variant 2).
-// The first radix is the largest (its products round at the finest scale); the
-// following ones are at most 8 where that keeps every shift <= kFxMaxShift
-// without giving up bits of S1.
+// A large first radix costs bits of S1, which shows with a spike over a small
+// background: with 16 instead of 8 at N = 1024 a spike at N/2 over 10^-3 had 1.1
+// times the error of FP64 butterflies (now 0.5), with 8 instead of 4 at 8192 a
+// spike anywhere over it 0.9 times (0.6).
 __host__ __device__ constexpr int fix_lanes(int N, int variant) {
   return N <= 8 ? 1 : N == 16 ? 4 : N == 32 ? 8 : N == 64 ? 16 : N == 128 ? (variant ? 32 : 16)
          : N == 256 ? (variant ? 64 : 32) : N <= 1024 ? (variant == 2 ? 128 : 64) : N <= 4096 ? 256 : 512;
@@ -337,11 +375,11 @@ template <> struct FixShape<256, 32> { enum { NP = 3, R0 = 8, R1 = 8, R2 = 4, R3
 template <> struct FixShape<256, 64> { enum { NP = 4, R0 = 4, R1 = 4, R2 = 4, R3 = 4 }; };
 template <> struct FixShape<512, 64> { enum { NP = 3, R0 = 8, R1 = 8, R2 = 8, R3 = 1 }; };
 template <> struct FixShape<512, 128> { enum { NP = 4, R0 = 8, R1 = 4, R2 = 4, R3 = 4 }; };
-template <> struct FixShape<1024, 64> { enum { NP = 3, R0 = 16, R1 = 8, R2 = 8, R3 = 1 }; };
+template <> struct FixShape<1024, 64> { enum { NP = 3, R0 = 8, R1 = 8, R2 = 16, R3 = 1 }; };
 template <> struct FixShape<1024, 128> { enum { NP = 4, R0 = 8, R1 = 8, R2 = 4, R3 = 4 }; };
 template <> struct FixShape<2048, 256> { enum { NP = 4, R0 = 8, R1 = 8, R2 = 8, R3 = 4 }; };
 template <> struct FixShape<4096, 256> { enum { NP = 3, R0 = 16, R1 = 16, R2 = 16, R3 = 1 }; };
-template <> struct FixShape<8192, 512> { enum { NP = 4, R0 = 16, R1 = 8, R2 = 8, R3 = 8 }; };
+template <> struct FixShape<8192, 512> { enum { NP = 4, R0 = 4, R1 = 8, R2 = 16, R3 = 16 }; };
 
 __host__ __device__ constexpr int fx_log2(int v) {
   int l = 0;
@@ -349,29 +387,73 @@ __host__ __device__ constexpr int fx_log2(int v) {
   return l;
 }
 
-// the scale plan of a shape: S1 and the shifts
+// the scale plan of a line of up to 1024 points: S1 and the shifts
 template <int R0, int R1, int R2, int R3>
 struct FixScale {
-  enum {
-    W0 = fx_log2(R0), W1 = fx_log2(R1), W2 = fx_log2(R2), W3 = fx_log2(R3),
-    // bits by which a radix above 8 would exceed kFxMaxShift, taken from S1
-    X = (W1 > 3 ? W1 - 3 : 0) + (W2 > 3 ? W2 - 3 : 0) + (W3 > 3 ? W3 - 3 : 0),
-    S1 = 61 - W0 - X
-  };
+  enum { W0 = fx_log2(R0), W1 = fx_log2(R1), W2 = fx_log2(R2), W3 = fx_log2(R3), S1 = 62 - W0 };
   // right shift, in all, of the values that enter pass p = 1 .. NP-1 (and are
   // twiddled there); 2^lb bounds the line's sum of |re| + |im| at the scale of
   // S1.  A pass shifts by at most kFxMaxShift, so a pass before the last takes
-  // more than its own bound asks for where the later ones could not.
+  // more than its own bound asks for where the later ones could not.  A last
+  // radix of 16 can need one bit more: it drops that one after two stages.
   template <int NP>
   static __host__ __device__ __forceinline__ int shift_at(int p, int lb) {
-    int all = S1 + 1 + W0 + W1 + W2 + W3, own = S1 + 1 + W0 + W1 + (p >= 2 ? W2 : 0) + (p >= 3 ? W3 : 0);
+    int all = S1 + W0 + W1 + W2 + W3, own = S1 + W0 + W1 + (p >= 2 ? W2 : 0) + (p >= 3 ? W3 : 0);
     all = (all < lb ? all : lb) - 62;
     own = (own < lb ? own : lb) - 62;
-    const int rest = all - kFxMaxShift * (NP - 1 - p);
+    const int rest = all - kFxMaxShift * (NP - 1 - p) - (p < NP - 1 && W2 > 3);
     own = own > rest ? own : rest;
     return own > 0 ? own : 0;
   }
+  // every shift and drop is within its limit
+  static constexpr bool kFits = W1 <= 3 && W2 <= (R3 > 1 ? 3 : 4) && W3 <= 3;
 };
+
+// The scale plan of a staged line.  |re|, |im| < 2^60 at the start of a pass, so
+// |z| < 2^60.5, 2^62.5 after two radix-2 stages, and below 2^62.5 again after all
+// four of a radix 16 that drops two bits in between.  The line's sum bounds every
+// value by 2^(lb-t), so from t = need on, where that is 2^62, nothing has to be
+// shifted any more; and t must end there, for the results' sake.
+template <int R0, int R1, int R2, int R3>
+struct FixStaged {
+  enum { S1 = 60, NEED = fx_log2(R0) + fx_log2(R1) + fx_log2(R2) + fx_log2(R3) + S1 - 62 };
+  // a component of the results is at most N 2^S1 2^-t: NEED is always enough
+  static __host__ __device__ __forceinline__ int need(int lb) {
+    const int n = lb - 62 < (int)NEED ? lb - 62 : (int)NEED;
+    return n > 0 ? n : 0;
+  }
+  // bits that radix r drops at most
+  static __host__ __device__ constexpr int head(int r) { return r >= 8 ? fx_log2(r) - 2 : 0; }
+  static __host__ __device__ __forceinline__ int drop(int r, int need, int t) {
+    const int d = need - t;
+    return d < 0 ? 0 : d < head(r) ? d : head(r);
+  }
+  // shift at the start of pass p = 1 .. NP-1, by -kFxMaxLeft to kFxMaxShift bits;
+  // top: OR of the high words of the values' magnitudes.  The last line: what the
+  // passes after this one's start could not make up for.
+  template <int NP>
+  static __host__ __device__ __forceinline__ int entry(int p, int need, int t, unsigned top) {
+#ifdef __CUDA_ARCH__
+    int sh = 64 - __clz((int)top) - 60;
+#else
+    int sh = (top ? 64 - __builtin_clz(top) : 32) - 60;
+#endif
+    sh = sh < need - t ? sh : need - t;
+    sh = sh > -kFxMaxLeft ? sh : -kFxMaxLeft;
+    const int later = kFxMaxShift * (NP - 1 - p) + head(R3) + (p <= 2 ? head(R2) : 0) + (p <= 1 ? head(R1) : 0);
+    const int least = need - t - later;
+    return sh > least ? sh : least;
+  }
+  // the passes together can always reach `need`
+  static constexpr bool kFits =
+      kFxMaxShift * ((R1 > 1) + (R2 > 1) + (R3 > 1)) + head(R0) + head(R1) + head(R2) + head(R3) >= (int)NEED;
+};
+// high word of |v| (of -v - 1 below zero)
+__host__ __device__ __forceinline__ unsigned fx_top(long long v) {
+  const int h = (int)(v >> 32);
+  return (unsigned)(h ^ (h >> 31));
+}
+__host__ __device__ constexpr bool fix_staged(int N) { return N >= 2048; }
 
 // entries of the pass tables [q][k] = w_{Ls r}^{q k}, passes 2 .. NP
 template <typename S>
@@ -410,7 +492,10 @@ template <int N, int TPL>
 struct FixLine {
   typedef FixShape<N, TPL> S;
   typedef FixScale<S::R0, S::R1, S::R2, S::R3> SC;
-  enum { NL = N / TPL, H = N / 2, CH = H / TPL, NW = TPL / 32, S1 = SC::S1,
+  typedef FixStaged<S::R0, S::R1, S::R2, S::R3> ST;
+  static constexpr bool kStaged = fix_staged(N);
+  static_assert(kStaged ? (bool)ST::kFits : (bool)SC::kFits, "shifts");
+  enum { NL = N / TPL, H = N / 2, CH = H / TPL, NW = TPL / 32, S1 = kStaged ? (int)ST::S1 : (int)SC::S1,
          // bits dropped from the magnitudes' high words so that their sum over
          // the line fits in 32 bits
          G = (S1 - 32) + fx_log2(2 * N) - 31 > 0 ? (S1 - 32) + fx_log2(2 * N) - 31 : 0 };
@@ -436,8 +521,19 @@ struct FixLine {
     return v;
   }
 
-  template <int R, int LSP, bool FIRST>
-  static __device__ __forceinline__ void pass(fx2* a, int t, const fxw* tp, int sh) {
+  // OR over the line's warps of what a pass left in their slots
+  static __device__ __forceinline__ unsigned line_or(const unsigned* slot) {
+    unsigned v = 0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) v |= slot[w];
+    return v;
+  }
+
+  // one pass; sh, drop: see FixScale and FixStaged.  TOP: leaves the OR of fx_top
+  // over the results in slot, one word a warp.
+  template <int R, int LSP, bool FIRST, bool TOP = false>
+  static __device__ __forceinline__ void pass(fx2* a, int t, const fxw* tp, int sh, unsigned drop = 0,
+                                              unsigned* slot = nullptr) {
     constexpr int GR = N / R, PER = (GR + TPL - 1) / TPL;
     const bool active = GR >= TPL || t < GR;  // a radix above N / TPL leaves lanes idle in its pass
     fx2 x[PER][R];
@@ -455,13 +551,24 @@ struct FixLine {
             // exact roots (k = 0) leave ties: rounded up and down in turn
             v = fx_cmul(tp[q * LSP + k], v, s, rnd - (q & 1));
           } else {
-            v.x = fx_shift(v.x, sh);
-            v.y = fx_shift(v.y, sh);
+            v.x = kStaged ? fx_rescale(v.x, sh) : fx_shift(v.x, sh);
+            v.y = kStaged ? fx_rescale(v.y, sh) : fx_shift(v.y, sh);
           }
         }
         x[i][q] = v;
       }
-      fx_dft<R>(x[i]);
+      fx_dft<R, kStaged || (!FIRST && R == 16)>(x[i], drop);
+    }
+    if constexpr (TOP) {
+      static_assert(GR >= TPL && TPL >= 32, "every lane of the warp has values");
+      unsigned top = 0;
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {
+#pragma unroll
+        for (int q = 0; q < R; ++q) top |= fx_top(x[i][q].x) | fx_top(x[i][q].y);
+      }
+      top = __reduce_or_sync(0xffffffffu, top);
+      if ((t & 31) == 0) slot[t >> 5] = top;
     }
     fx_line_sync(TPL);
 #pragma unroll
@@ -473,6 +580,17 @@ struct FixLine {
         a[LSP == 1 && R % 8 == 0 ? fpad(j * R) + fpad(q) : fpad_step<LSP>(j * LSP * R + k, q)] = x[i][q];
     }
     fx_line_sync(TPL);
+  }
+
+  // lb: 2^lb bounds the line's sum of |re| + |im|; sum: its G-bit part, of the
+  // lane's line (up to 32 lanes) or of each warp, in slot
+  static __device__ __forceinline__ int sum_bits(const unsigned* slot, unsigned sum) {
+    if constexpr (TPL > 32) {
+      sum = 0;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) sum += slot[w];
+    }
+    return 32 + G + 32 - __clz(sum + 2 * N);
   }
 
   // Unnormalised DST-I of the line (doubles at fpad(1) .. fpad(N-1)) in place.
@@ -530,28 +648,46 @@ struct FixLine {
         for (int d = 1; d < TPL; d <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d, TPL);
       }
       fx_line_sync(TPL);
-      pass<S::R0, 1, true>(a, t, tp, 0);
-      if constexpr (TPL > 32) {
-        sum = 0;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) sum += s_sum[w];
+      if constexpr (kStaged) {
+        const int lb = sum_bits(s_sum, sum);
+        const int need = ST::need(lb);
+        int d = ST::drop(S::R0, need, 0), all = d, sh;
+        pass<S::R0, 1, true, true>(a, t, tp, 0, d, s_max);
+        sh = ST::template entry<S::NP>(1, need, all, line_or(s_max));
+        d = ST::drop(S::R1, need, all + sh);
+        all += sh + d;
+        pass<S::R1, S::R0, false, true>(a, t, tp, sh, d, s_max);
+        tp += S::R0 * S::R1;
+        sh = ST::template entry<S::NP>(2, need, all, line_or(s_max));
+        d = ST::drop(S::R2, need, all + sh);
+        all += sh + d;
+        pass<S::R2, S::R0 * S::R1, false, (S::NP > 3)>(a, t, tp, sh, d, s_max);
+        if constexpr (S::NP > 3) {
+          tp += S::R0 * S::R1 * S::R2;
+          sh = ST::template entry<S::NP>(3, need, all, line_or(s_max));
+          d = ST::drop(S::R3, need, all + sh);
+          all += sh + d;
+          pass<S::R3, S::R0 * S::R1 * S::R2, false>(a, t, tp, sh, d);
+        }
+        E += all;
+      } else {
+        pass<S::R0, 1, true>(a, t, tp, 0);
+        const int lb = sum_bits(s_sum, sum);
+        int t1 = 0, tn = SC::template shift_at<S::NP>(1, lb);
+        pass<S::R1, S::R0, false>(a, t, tp, tn);
+        if constexpr (S::NP > 2) {
+          t1 = tn;
+          tn = SC::template shift_at<S::NP>(2, lb);
+          const int d = S::R2 == 16 && tn - t1 > kFxMaxShift ? 1 : 0;
+          pass<S::R2, S::R0 * S::R1, false>(a, t, tp + S::R0 * S::R1, tn - t1 - d, d);
+        }
+        if constexpr (S::NP > 3) {
+          t1 = tn;
+          tn = SC::template shift_at<S::NP>(3, lb);
+          pass<S::R3, S::R0 * S::R1 * S::R2, false>(a, t, tp + S::R0 * S::R1 + S::R0 * S::R1 * S::R2, tn - t1);
+        }
+        E += tn;
       }
-      sum += 2 * N;
-      const int lb = 32 + G + 32 - __clz(sum);
-      int t1 = 0, tn = 0;
-      tn = SC::template shift_at<S::NP>(1, lb);
-      pass<S::R1, S::R0, false>(a, t, tp, tn);
-      if constexpr (S::NP > 2) {
-        t1 = tn;
-        tn = SC::template shift_at<S::NP>(2, lb);
-        pass<S::R2, S::R0 * S::R1, false>(a, t, tp + S::R0 * S::R1, tn - t1);
-      }
-      if constexpr (S::NP > 3) {
-        t1 = tn;
-        tn = SC::template shift_at<S::NP>(3, lb);
-        pass<S::R3, S::R0 * S::R1 * S::R2, false>(a, t, tp + S::R0 * S::R1 + S::R0 * S::R1 * S::R2, tn - t1);
-      }
-      E += tn;
     }
     post.start();
     // ---- split into C_k and S_k and prefix sum of C: the lane's chunk k = CH t + i
@@ -606,7 +742,7 @@ struct FixLine {
 // lines of 4 or 8 points: the whole line in one lane's registers
 template <int N>
 struct FixLine<N, 1> {
-  enum { S1 = 61 - fx_log2(N) };
+  enum { S1 = 62 - fx_log2(N) };
   template <typename POST>
   static __device__ __forceinline__ void run(double2* line, int, const int2* hs, const fxw*, void*, POST& post) {
     unsigned mx = 0;
