@@ -89,7 +89,8 @@ typedef enum csl_precision {
 typedef struct csl_plan_options {
   int precision;          /* csl_precision, default CSL_PREC_FP64                          */
   double gamma_override;  /* > 0: use this gamma in P; otherwise sqrt(min a * max a) (Eq. 4) */
-  int lines_per_cta;      /* sine-transform lines per CTA for the strided passes; 0 = tuned */
+  int lines_per_cta;      /* sine-transform lines per CTA for the strided passes (rounded up to
+                             a power of two, at most what 256 threads hold); 0 = tuned */
   int use_graph;          /* 1 (default): the iteration loop runs as a CUDA graph with a
                              device-controlled WHILE node; 0: host-driven loop              */
   int autotune;           /* 1 (default): time the candidate CTA shapes and transform

@@ -333,10 +333,10 @@ void config_strided(PassCfg& c, int n, int ncols, int nouter, long outer_stride,
   const int tpl = pass_tpl<T>(c.N, c.wide);
   int threads = 256;
   if (want_lines > 0) {
+    // the kernels are compiled for CTAs of up to 256 threads (pass_max_threads)
     int l = 1;
-    while (l < want_lines) l <<= 1;
+    while (l < want_lines && l * tpl < 256) l <<= 1;
     threads = l * tpl < 32 ? 32 : l * tpl;
-    if (threads > 1024) threads = 1024;
   }
   // no wider than the grid's x extent needs
   while (threads > 32 && threads > tpl && (threads / tpl) / 2 >= ncols) threads >>= 1;
