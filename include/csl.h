@@ -369,7 +369,9 @@ size_t csl_batch_workspace_bytes(const csl_batch* batch);
  * shared by all calls: calls that overlap on the GPU race and must be
  * serialised by the caller.  Every call rewrites all the scratch it reads.
  * The first call on a device performs a one-time set-up: it looks up the
- * arrays' device addresses (cudaGetSymbolAddress) with that device current.
+ * arrays' device addresses (cudaGetSymbolAddress) with that device current;
+ * the first call of a precision and line length sets its kernels' shared-memory
+ * limit (cudaFuncSetAttribute).
  */
 csl_status csl_precondition_static(int dim, const int64_t n[3], double gamma, double alpha, double beta,
                                    int precision, const double* v, double* out, void* stream);

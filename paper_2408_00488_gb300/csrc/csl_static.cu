@@ -12,7 +12,9 @@
 // intermediate it reads, so nothing needs clearing between calls.
 //
 // Set-up: the first call on a device looks up the device addresses of the
-// arrays (cudaGetSymbolAddress) with that device current.
+// arrays (cudaGetSymbolAddress) with that device current, and the first call
+// of a precision and line length there lets its kernels take the shared memory
+// that their tiles need (plans do it for all kernels when the first is created).
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -55,6 +57,8 @@ struct StaticPtrs {
 StaticPtrs g_ptrs[kMaxDevices];
 std::once_flag g_once[kMaxDevices];
 cudaError_t g_setup_err[kMaxDevices];
+std::mutex g_attr_mu;
+bool g_attr_set[kMaxDevices][2][16];  // by device, FP64, log2 of the line length
 
 int ilog2_exact_s(long v) {
   if (v <= 0 || (v & (v - 1))) return -1;
@@ -170,6 +174,23 @@ void setup_device(int dev) {
   if (e == cudaSuccess) e = cudaGetSymbolAddress((void**)&p.tables, g_static_tables);
   g_ptrs[dev] = p;
   g_setup_err[dev] = e;
+}
+
+// opt-in shared memory of the pass kernels of length N (static_launch's variant)
+template <typename T>
+cudaError_t allow_static_smem(int dev, int N) {
+  std::lock_guard<std::mutex> lk(g_attr_mu);
+  bool& set = g_attr_set[dev][sizeof(T) == 8][ilog2_exact_s(N)];
+  if (set) return cudaSuccess;
+  cudaError_t e = cudaErrorInvalidValue;
+  switch (N) {
+#define CASE(NN) \
+  case NN: e = set_pass_attrs_n<T, NN, (NN >= 512 ? 1 : 0)>(); break;
+    CSL_FOR_EACH_N(CASE)
+#undef CASE
+  }
+  set = e == cudaSuccess;
+  return e;
 }
 
 // CTA shape of one pass (same rules as the plan's default configuration)
@@ -363,6 +384,13 @@ extern "C" csl_status csl_precondition_static(int dim, const int64_t n[3], doubl
   std::call_once(g_once[dev], setup_device, dev);
   if (g_setup_err[dev] != cudaSuccess) {
     csl_internal_set_error("csl_precondition_static: cudaGetSymbolAddress failed during set-up");
+    return CSL_CUDA_ERROR;
+  }
+  for (int d = 0; d < dim && e == cudaSuccess; ++d)
+    e = precision == CSL_PREC_FP32 ? allow_static_smem<float>(dev, nn[d] + 1) : allow_static_smem<double>(dev, nn[d] + 1);
+  if (e != cudaSuccess) {
+    (void)cudaGetLastError();
+    csl_internal_set_error("csl_precondition_static: cudaFuncSetAttribute failed during set-up");
     return CSL_CUDA_ERROR;
   }
   e = (precision == CSL_PREC_FP32)
