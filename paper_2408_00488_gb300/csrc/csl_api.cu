@@ -60,7 +60,7 @@ const double kNaN = __builtin_nan("");
 // one sine-transform pass: line length N = n + 1, CTA shape and grid
 struct PassCfg {
   int N = 0, n = 0, lines = 0;  // lines per CTA
-  int wide = 0;                  // N = 512, 1024: 0 warp per line, 1 / 2 Stockham with 64 / 128 lanes per line
+  int wide = 0;                  // the kernels' variant (pass_num_variants), 3 long lines, 4 two-CTA clusters
   int ncols = 0, nouter = 0;     // strided: x extent and outer blocks; row: nouter = rows
   long outer_stride = 0, line_stride = 0;
   PassLaunch L = {1, 32, 0};
@@ -1429,17 +1429,23 @@ csl_status csl_plan_create(csl_plan** out, int dim, const int64_t n[3], const do
                                                                 : "bf16x6";
     int off = snprintf(P->config, sizeof(P->config), "%s%s stencil[%s strip=%d blocks=%d]", pname,
                        o.autotune ? " autotuned" : "", P->ff ? "float-pair" : "fp64", P->sten_strip, P->sten_blocks);
-    for (int d = 0; d < dim && off < (int)sizeof(P->config); ++d)
+    for (int d = 0; d < dim && off < (int)sizeof(P->config); ++d) {
+      char kernel[48];
+      if (fp64 && cs[d]->wide < 4)  // lanes per line: the threads divided by the lines
+        snprintf(kernel, sizeof(kernel), "%sfixed-point%d", cs[d]->wide == 3 ? "long-line " : "",
+                 pass_tpl<double>(cs[d]->N, cs[d]->wide));
+      else
+        snprintf(kernel, sizeof(kernel), "%s",
+                 cs[d]->L.tc == 2   ? "tcgen05-bf16x3"
+                 : cs[d]->L.tc == 3 ? "tcgen05-bf16x6"
+                 : cs[d]->wide == 4 ? "cluster2"
+                 : cs[d]->wide == 3 ? "long-line"
+                 : cs[d]->wide == 2 ? "stockham128"
+                 : cs[d]->wide == 1 ? "stockham64"
+                                    : "warp");
       off += snprintf(P->config + off, sizeof(P->config) - off, " %s[N=%d %s lines=%d threads=%d blocks=%d smem=%zu]",
-                      nm[d], cs[d]->N,
-                      cs[d]->L.tc == 2   ? "tcgen05-bf16x3"
-                      : cs[d]->L.tc == 3 ? "tcgen05-bf16x6"
-                      : cs[d]->wide == 4 ? "cluster2"
-                      : cs[d]->wide == 3 ? "long-line"
-                      : cs[d]->wide == 2 ? "stockham128"
-                      : cs[d]->wide == 1 ? "stockham64"
-                                         : "warp",
-                      cs[d]->lines, cs[d]->L.threads, cs[d]->L.blocks, cs[d]->L.smem);
+                      nm[d], cs[d]->N, kernel, cs[d]->lines, cs[d]->L.threads, cs[d]->L.blocks, cs[d]->L.smem);
+    }
   }
   *out = P;
   return CSL_OK;
