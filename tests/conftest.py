@@ -14,6 +14,9 @@ def pytest_configure(config):
 
 
 def pytest_collection_modifyitems(config, items):
+    # test_variants loads forced shapes into the process-wide cache of tuned shapes: it runs last, so
+    # that every other test has the shapes that a user's plan gets
+    items.sort(key=lambda it: getattr(it, "originalname", None) == "test_variants")
     try:
         import torch
         has_gpu = torch.cuda.is_available()
