@@ -734,12 +734,14 @@ DevState scratch_state(const csl_plan* P) {
 }
 
 // ---- autotuner ---------------------------------------------------------------
-// Each sine-transform pass tries every CTA size and, for N = 512 and 1024,
-// every transform variant.  A candidate is timed inside the iteration's own
-// kernel sequence (time_sequence: three iterations after a warm-up, on
-// zeroed vectors and a scratch state, the MID pass with its reduction but
-// without the Givens step),
-// so that its cost includes the caches and the predecessor it really has;
+// Each sine-transform pass tries every CTA size (but for the narrowest tiles,
+// see tune_pass) and, for N = 512 and 1024, in FP64 also 128 and 256, every
+// transform variant.  A candidate is timed inside the iteration's own kernel
+// sequence (time_sequence: three iterations after a warm-up, on zeroed vectors
+// and a scratch state, the MID pass with its reduction but without the Givens
+// step), so that its cost includes the caches and the predecessor it really has.
+// In FP64 the zeroed vectors take the far case of fx_to_double in every store,
+// which solves do not take, the same for each candidate of a pass;
 // the candidate with the smallest summed duration of the pass's kernels is
 // kept.  Results are cached per (precision, pass, geometry) for the life of
 // the process, and can be saved to and loaded from a file.
@@ -758,7 +760,8 @@ std::mutex g_tune_mu;
 
 // One candidate shape of a pass: transform variant w with `lines` lines per
 // CTA; false when the shape is not allowed (CTA size, shared memory, tile
-// wider than twice the grid's x extent).  Used by the tuner and by the cache
+// wider than twice the grid's x extent).  In FP64 at N >= 512 variant 0 of an
+// older file means variant 1.  Used by the tuner and by the cache
 // loader, so a shape read from a file is rebuilt and checked the same way.
 template <typename T>
 bool make_candidate(const PassCfg& c, int kind, int w, int lines, PassCfg& cand) {

@@ -486,9 +486,8 @@ struct LineDst {
 // Long lines (N = 2048 .. 8192, 2D grids of the paper's large tables): one
 // CTA of TPL lanes per line, an NP-pass Stockham autosort FFT (radices R0..R3)
 // whose inter-pass twiddles w_{Ls r}^{q k} = w_N^{q k N/(Ls r)} come from the
-// length-N table itself, so no per-pass tables exist; the line (up to 128 KB
-// in FP64) fills shared memory and the tables are read from global memory
-// through the cache.  Pre-twiddle, split and prefix scan as in the wide path.
+// length-N table itself, so no per-pass tables exist; the tables are read from
+// global memory through the cache.  FP32 only (the FP64 form: csl_fix.cuh).  Pre-twiddle, split and prefix scan as in the wide path.
 // ---------------------------------------------------------------------------
 template <int N> struct BigShape;
 template <> struct BigShape<2048> { enum { TPL = 256, NP = 3, R0 = 8, R1 = 16, R2 = 16, R3 = 1 }; };
@@ -644,7 +643,7 @@ struct FixDst {
   static __device__ __forceinline__ int in_pos(int j) { return fpad(j); }
   static __device__ __forceinline__ int out_pos(int m) { return fpad(m); }
   // scr: SCRATCH slots per line
-  template <bool PERM_IN>
+  template <bool>  // input and output positions agree
   static __device__ __forceinline__ void run(double2* a, int t, const Tab& tb, double2* scr) {
     FixNoPost none;
     run_post(a, t, tb, scr, none);

@@ -340,8 +340,8 @@ static __device__ __noinline__ double fx_scale_far(double d, int q) { return sca
 
 // v * 2^q.  The hardware conversion rounds to nearest (one FP64-pipe
 // operation); the exponent is added with integer instructions.  The far case
-// stays a call: inlined, its products would be issued on the FP64 pipe for
-// every value and discarded.
+// (zero lines, and lines near the ends of the range) stays a call: inlined, its
+// products would be issued on the FP64 pipe for every value and discarded.
 __device__ __forceinline__ double fx_to_double(long long v, int q) {
   const double d = __ll2double_rn(v);
   if (q < -1000 || q > 900) return fx_scale_far(d, q);

@@ -881,8 +881,9 @@ __device__ inline void givens_step(DevState* st, double g2) {
 // hold w scaled by its a1, so w_a = 1) over w_{j-1}'s buffer, and
 // x_j = x_{j-1} + x_coef w_{j+1}; the coefficients come from the Givens step
 // in the MID pass.  Per point: ẑ_j, w_{j-1}, w_j, x read, w_{j+1}, x written.
-// w and x are read once an iteration and by this kernel alone, so they are
-// loaded and stored evict-first: at n = 1023 the other vectors and the faces
+// w is read once an iteration and by this kernel alone, x by it and by the few
+// stencil passes that check the residual, so they are loaded and stored
+// evict-first: at n = 1023 the other vectors and the faces
 // (75 MB in the pair form) then stay in the 129 MB L2, and the x pass that
 // follows the stencil falls from 20.0 to 16.5 us, the iteration from 82.1 to
 // 76.9.

@@ -1,7 +1,7 @@
-// Launch wrappers of the sine-transform passes for one real type and one
-// length (launch_*_n), and, where CSL_T is defined, the dispatch over the
-// lengths.  csl_pass32.cu holds every FP32 length; the FP64 ones are spread
-// over csl_pass64*.cu so that they compile in parallel.
+// Launch wrappers of the sine-transform passes for one real type, length and
+// variant (launch_*_n).  csl_pass32.cu holds every FP32 length; the FP64 ones are
+// spread over csl_pass64*.cu so that they compile in parallel.  The dispatch over
+// the lengths is csl_pass_dispatch.cu.
 #pragma once
 #include "csl_passes.cuh"
 

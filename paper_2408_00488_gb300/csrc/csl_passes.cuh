@@ -93,8 +93,6 @@ __host__ __device__ constexpr int pass_max_threads() {
   return WIDE == 3 ? (N >= 8192 ? 512 : 256) : 256;
 }
 
-__device__ __forceinline__ float rsq(float v) { return rsqrtf(v); }
-__device__ __forceinline__ double rsq(double v) { return rsqrt(v); }
 
 template <typename T, int N, int WIDE, int LOAD_MODE, int STORE_MODE>
 __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_ROW_MINB(T, N, WIDE, LOAD_MODE, STORE_MODE))
@@ -394,7 +392,6 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_PASS_MINB(T, 
   const StridedArgs<T> a = batch ? batch[sys] : a0;
   constexpr int TPL = D::TPL, LS = D::LS;
   constexpr int NL = (N + TPL - 1) / TPL;
-  constexpr int UB = NL < 8 ? NL : 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int C = blockDim.x / TPL;  // lines (columns) per tile, a power of two
   c_t* s_scr = (c_t*)(smem_raw + D::Tables::kBytes);
@@ -474,7 +471,7 @@ __global__ void __launch_bounds__(pass_max_threads<N, WIDE>(), CSL_PASS_MINB(T, 
             const int pos = D::out_pos(m);
             c_t F = line[pos];
             const T e = fma(a.gamma, murest + mu[k], a.alpha);
-            const T sc = a.cnorm * rsq(fma(e, e, a.beta2));
+            const T sc = a.cnorm * rsqrtf(fma(e, e, a.beta2));
             part = fma(sc, fma(F.x, F.x, F.y * F.y), part);
             F.x *= sc;
             F.y *= sc;
