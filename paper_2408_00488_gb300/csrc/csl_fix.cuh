@@ -169,11 +169,15 @@ __host__ __device__ __forceinline__ long long fx_take(long long acc, long long m
 #endif
 }
 
-// v * w for real v and a constant of F fractional bits (digits h, l), rounded
+// v * w for real v and a constant of F fractional bits (digits h, l), rounded.
+// The product of the two low digits, at most 2^(62-F) units, only for the half
+// sines (F = 62): with it the error of a spike over 10^-3 is 0.7 times that without
+// at N = 8192.  For the diagonal roots (F = 63) it made no difference.
 template <int F>
 __host__ __device__ __forceinline__ long long fx_rmul(long long v, int h, int l) {
   const int vh = fx_hi(v), vl = fx_lo(v);
-  const long long mid = (1ll << (F - 33)) + (fx_wide(vl, l) >> 32) + fx_wide(vh, l) + fx_wide(vl, h);
+  long long mid = (1ll << (F - 33)) + fx_wide(vh, l) + fx_wide(vl, h);
+  if (F < 63) mid += fx_wide(vl, l) >> 32;
   return fx_take(fx_wide(vh, h) + (mid >> 32), mid, F - 32);
 }
 
