@@ -33,9 +33,9 @@
 //
 // Measured on a GB300, FP64 form, per iteration of MINRES, FP64 arithmetic and
 // this (with the lanes of fix_lanes and the tables in the L1): n = 1023 in 2D, x
-// pass with the Lanczos step 124.6 and 33.9 us, MID pass 252.5 and 66.7, inverse
-// x pass 119.0 and 27.2, whole iteration 524 and 166; n = 63, 71 and 35 us;
-// n = 127 in 3D 1067 and 360; n = 4095 9297 and 2553.  Error of one
+// pass with the Lanczos step 124.6 and 33.4 us, MID pass 252.5 and 69.1, inverse
+// x pass 119.0 and 27.9, whole iteration 524 and 168; n = 63, 71 and 35 us;
+// n = 127 in 3D 1067 and 360; n = 4095 9297 and 2680.  Error of one
 // line against 64-bit mantissas or more, over that of FP64 butterflies with the
 // same split and scan, root mean square over 96 lines of a kind (random, constant,
 // alternating, one to eight spikes anywhere or at N/2 and N/4 over random and
@@ -170,14 +170,15 @@ __host__ __device__ __forceinline__ long long fx_take(long long acc, long long m
 }
 
 // v * w for real v and a constant of F fractional bits (digits h, l), rounded.
-// The product of the two low digits, at most 2^(62-F) units, only for the half
-// sines (F = 62): with it the error of a spike over 10^-3 is 0.7 times that without
-// at N = 8192.  For the diagonal roots (F = 63) it made no difference.
-template <int F>
+// LOW: with the product of the two low digits, at most 2^(62-F) units.  The half
+// sines of long lines take it: the error of a spike over 10^-3 is 0.7 times that
+// without at N = 8192, 0.8 at 1024.  At 512, where it is a third of FP64's anyway, it
+// cost the 3D P^-1 2%; for the diagonal roots (F = 63) it made no difference.
+template <int F, bool LOW = false>
 __host__ __device__ __forceinline__ long long fx_rmul(long long v, int h, int l) {
   const int vh = fx_hi(v), vl = fx_lo(v);
   long long mid = (1ll << (F - 33)) + fx_wide(vh, l) + fx_wide(vl, h);
-  if (F < 63) mid += fx_wide(vl, l) >> 32;
+  if (LOW) mid += fx_wide(vl, l) >> 32;
   return fx_take(fx_wide(vh, h) + (mid >> 32), mid, F - 32);
 }
 
@@ -497,7 +498,7 @@ struct FixLine {
   typedef FixShape<N, TPL> S;
   typedef FixScale<S::R0, S::R1, S::R2, S::R3> SC;
   typedef FixStaged<S::R0, S::R1, S::R2, S::R3> ST;
-  static constexpr bool kStaged = fix_staged(N);
+  static constexpr bool kStaged = fix_staged(N), kLow = N >= 1024;
   static_assert(kStaged ? (bool)ST::kFits : (bool)SC::kFits, "shifts");
   enum { NL = N / TPL, H = N / 2, CH = H / TPL, NW = TPL / 32, S1 = kStaged ? (int)ST::S1 : (int)SC::S1,
          // bits dropped from the magnitudes' high words so that their sum over
@@ -635,7 +636,7 @@ struct FixLine {
         sum += ((g0 >> G) + (g1 >> G)) + ((g2 >> G) + (g3 >> G));
         const int2 h = hs[1 + t + TPL * i];
         const fx2 p = fx_add(u, v), d = fx_sub(u, v);
-        const fx2 A = {fx_rmul<62>(p.x, h.x, h.y), fx_rmul<62>(p.y, h.x, h.y)};
+        const fx2 A = {fx_rmul<62, kLow>(p.x, h.x, h.y), fx_rmul<62, kLow>(p.y, h.x, h.y)};
         // the quarter, ties rounded up and down in turn
         const fx2 B = {(d.x + 1 + (i & 1)) >> 2, (d.y + 1 + (i & 1)) >> 2};
         a[fpad_step<TPL>(1 + t, i)] = fx_add(A, B);

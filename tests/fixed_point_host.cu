@@ -201,7 +201,8 @@ static std::vector<Cd> fixed(const std::vector<Cd>& z) {
   for (int j = 1; j <= N / 2; ++j) {
     const int2 h = fx_half_sine(j, N);
     const fx2 p = fx_add(a[j], a[N - j]), d = fx_sub(a[j], a[N - j]);
-    const fx2 A = {fx_rmul<62>(p.x, h.x, h.y), fx_rmul<62>(p.y, h.x, h.y)};
+    constexpr bool LOW = FixLine<N, LANES>::kLow;
+    const fx2 A = {fx_rmul<62, LOW>(p.x, h.x, h.y), fx_rmul<62, LOW>(p.y, h.x, h.y)};
     const int up = ((j - 1) / LANES) & 1;
     const fx2 B = {(d.x + 1 + up) >> 2, (d.y + 1 + up) >> 2};
     y[j] = fx_add(A, B);
