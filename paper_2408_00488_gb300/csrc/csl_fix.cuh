@@ -42,8 +42,9 @@
 // constant backgrounds of 10^-8 to 0.1, the modes of such lines;
 // tests/fixed_point_host.cu): at most 0.2 for N <= 256, 0.3 at 512, 0.5 at 1024, 0.4
 // at 2048, 0.7 at 4096 and 8192; random and constant lines 0.1 to 0.2.  A single
-// line can come out either way.  What bounds the time is latency: 13 to 20 warps
-// per SM (registers and shared memory hold the lines).
+// line can come out either way.  What bounds the time is latency: at n = 1023 14
+// warps per SM (the registers allow 16) keep the ALU 33 to 37% busy and issue in 38
+// to 41% of the cycles.
 //
 // A line with an infinity or NaN returns NaN everywhere (the FP64 butterflies
 // spread it over the line too); a zero line returns zeros.
