@@ -324,18 +324,18 @@ __device__ void mid_scalar_tail(const StridedArgs<T>& a, double g2acc, int bid, 
   // four lanes of the last CTA go on, each with the same state (givens_step)
   if (!grid_sum_last_block<1>(v, a.partials, &a.st->tickets[TICKET_MID], tot, bid, nblk)) return;
   if (threadIdx.x > 3 || a.scalar_mode == 3) return;  // 3: tuning: the cost of the reduction, not its result
-  // recorded by an earlier kernel or, after the copy `pre`, by a CTA of this one
-  // (ordered before this read by the CTA's arrival)
-  if (__ldcg(&a.st->timeout)) {
+  // the scalar step runs on a register copy of the state and stores the
+  // fields it sets
+  DevState q = pre ? *pre : *a.st;
+  // a time-out of an earlier kernel is in the copy; one of this kernel made the sum
+  // a NaN (the CTA's arrival orders it before this read)
+  if (q.timeout || (!(tot[0] == tot[0]) && __ldcg(&a.st->timeout))) {
     if (threadIdx.x == 0) {
       a.st->status = ST_TIMEOUT;
       a.st->done = 1;
     }
     return;
   }
-  // the scalar step runs on a register copy of the state and stores the
-  // fields it sets
-  DevState q = pre ? *pre : *a.st;
   if (a.scalar_mode == 1) {
     const double g2 = tot[0];
     // f = 0 never reaches this pass (the ingest closes the solve with z = 0),

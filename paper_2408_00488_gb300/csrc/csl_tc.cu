@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   tc_fence_before();
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS));
-  if (!ok && tid == 0 && a.st) record_timeout(a.st);
+  if (!ok && tid == 0 && a.st) g2acc += record_timeout(a.st);
   if (MID && a.scalar_mode != 0) mid_scalar_tail<float>(a, g2acc, bid, nblk, &s_pre);
 }
 
